@@ -47,7 +47,8 @@ ADMM_API long long admm_cnn_param_count(void);
  * admm_cnn_create -- allocate a network for batches of up to `max_pixels`
  * pixels in total (count x H x W). training = 1 also allocates what
  * admm_cnn_train_step and admm_cnn_gradients need (stored activations,
- * gradients, Adam moments: about 0.7 KB per pixel); 0 keeps inference only.
+ * gradients, Adam moments: about 0.7 KB per pixel, and one gradient vector
+ * per SM, 35 MB); 0 keeps inference only.
  * Parameters start at zero: set them with admm_cnn_set_params.
  * Errors: ADMM_EINVAL, ADMM_ENOMEM, ADMM_ECUDA.
  */

@@ -1,7 +1,7 @@
 // cnn.cu -- the learned warm start: a stack of 3 x 3 convolutions on BF16
 // tensor cores (tcgen05.mma, FP32 accumulate in tensor memory), its backward
-// pass (weight gradients on mma.sync m16n8k16) and Adam. Not part of the paper; Theorem 1 (convergence from any u0, d0) is
-// what lets a predicted start feed Algorithm 2.
+// pass and Adam. Not part of the paper; Theorem 1 (convergence from any u0,
+// d0) is what lets a predicted start feed Algorithm 2.
 //
 // Layout. Activations and their gradients are BF16 in planes of eight
 // channels: [image][C / 8][H][W][8], C padded to 8 (the network's input),
@@ -18,11 +18,8 @@
 // input gradients gated by the ReLU of the layer below, and the last layer
 // (4 outputs padded to 16) with bias into FP32.
 //
-// Weight-gradient kernel: per tap, dW_tap = G^T A_tap, a contraction over
-// pixels. A CTA of 9 warps (one per tap) loops over tiles; the gradient and
-// activation tiles are stored channel-major in shared memory so the MMA
-// operands are pixel pairs of one channel; the CTA's FP32 partial sums go to
-// global memory with one atomic add per element at the end.
+// The weight gradients are contractions over pixels, also on tcgen05
+// (conv3x3_wgrad_tc): both operands MN-major, straight from the same planes.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -80,17 +77,6 @@ int fail(cudaError_t) { return ADMM_ECUDA; }
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ uint32_t ld32(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
 __device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
@@ -215,8 +201,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 16 consecutive FP32 columns of this thread's accumulator lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+// 8 or 16 consecutive FP32 columns of this thread's accumulator lane
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
@@ -382,7 +379,7 @@ conv3x3_tc(const __grid_constant__ CUtensorMap tin, const bf16* __restrict__ wpk
         const uint32_t tacc = tmem + (uint32_t)COUT * b + ((uint32_t)(32 * warp) << 16);
         if constexpr (MODE == kModeOutF32) {
             float v[16];
-            tmem_ld16(tacc, v);
+            tmem_ld(tacc, v);
             const size_t px = (size_t)img * hw + (size_t)(y0 + oy) * W + (x0 + ox);
             reinterpret_cast<float4*>(out)[px] =
                 make_float4(v[0] + smB[0], v[1] + smB[1], v[2] + smB[2], v[3] + smB[3]);
@@ -438,121 +435,305 @@ conv3x3_tc(const __grid_constant__ CUtensorMap tin, const bf16* __restrict__ wpk
 }
 
 // ---------------------------------------------------------------------------
-// weight and bias gradients of one layer
-// a: [img][H][W][CIN] (layer input), g: [img][H][W][COUT] (gradient in the
-// layer's pre-activation output). dw: FP32 [cout_real][cin_real][9] slice of
-// the gradient vector, db: [cout_real].
+// weight and bias gradients of one layer on tcgen05
+//
+// Per tap, dW_tap = G^T A_tap is a contraction over pixels: K = 16 adjacent
+// pixels of one row per MMA, both operands MN-major (a pixel's eight channels
+// of one plane are 16 contiguous bytes, eight adjacent pixels one 128-byte core
+// matrix), so tiles go from memory to the tensor cores without a transpose.
+// TMA lands a tile as [row][plane][column][8 channels]: consecutive (row,
+// plane) pairs are one plane row apart, so one operand can span several image
+// rows with a single stride, and the taps' row offsets dy come out of one MMA:
+//   GA = false (32 input channels): A operand = 4 activation rows x 32 channels
+//     (M = 128), B operand = 2 gradient rows (N = 2 x 8 PG); block (ay, gy) of
+//     the accumulator belongs to dy = ay - gy, 6 of the 8 blocks are taps;
+//   GA = true (the first layer, one plane of inputs): A operand = 4 gradient
+//     rows x 32 channels, B operand = 6 activation rows (N = 48).
+// The column offset dx is a shifted start address: three accumulators. Per 32
+// pixels of a 32-channel layer: 3 MMAs of 128 x 64 x 16, 6 KB of shared-memory
+// reads each, 4.5 cycles per pixel and SM, under the 5.6 cycles that the
+// 128 B/pixel take from HBM.
+//
+// One CTA per SM walks tiles of 16 x 32 pixels (18 x 34 activation halo; what
+// lies outside the image reads as zero, so ragged tiles need no mask): lane 0
+// of warp 0 requests tiles three stages ahead, lane 0 of warp 1 issues the
+// MMAs, warps 2 and 3 sum the gradient tile for the bias. The accumulators
+// stay in tensor memory until the CTA's last tile; each CTA then stores one
+// partial gradient vector (layout [tap][cout][cin], then the bias), and
+// wgrad_reduce_kernel adds the CTAs' vectors in a fixed order.
+// 16 x 256^2, 32 x 32 channels: 34 us per launch (134 MB of activations and
+// gradients, 4.0 TB/s); 180 us with mma.sync on tiles transposed through
+// shared memory and one atomic per weight and CTA.
 // ---------------------------------------------------------------------------
-template <int CIN, int COUT>
+constexpr int kWgTW = 32, kWgTH = 16, kWgStages = 3;
+
+template <bool GA, int PA, int PG>
 struct WgradCfg {
-    static constexpr int HALO = kTile + 2;
-    static constexpr int PA = HALO * HALO + 4;       // activation plane stride (elements)
-    static constexpr int PG = kTile * kTile + 8;     // gradient plane stride
-    static constexpr size_t SMEM = (size_t)(CIN * PA + COUT * PG) * sizeof(bf16) + COUT * sizeof(float);
-    static_assert(SMEM <= 48 * 1024, "fits the default shared-memory window");
+    static constexpr int AW = kWgTW + 2, AR = kWgTH + 2;                  // activation tile with halo
+    static constexpr int ABYTES = AR * PA * AW * 16, GBYTES = kWgTH * PG * kWgTW * 16;
+    static constexpr int ASTRIDE = (ABYTES + 127) / 128 * 128;             // TMA destinations on 128 bytes
+    static constexpr int STAGE = ASTRIDE + GBYTES;
+    static constexpr int STEP = GA ? 4 : 2;                                // output rows per MMA
+    static constexpr int N = GA ? 8 * PA * (STEP + 2) : 8 * PG * STEP;     // accumulator columns per dx
+    static constexpr int TMEM_COLS = 3 * N <= 64 ? 64 : (3 * N <= 128 ? 128 : 256);
+    static constexpr int COUT = 8 * PG;
+    static_assert(GBYTES % 128 == 0 && N % 16 == 0 && 3 * N <= 256, "tile");
+    static_assert(GA ? PG == 4 : PA == 4, "the A operand spans 128 rows");
+    // epilogue scratch (reuses the stages): GA = false 9 COUT x 32 floats, GA =
+    // true 4 x 18 x 32; the bias sums of two warps follow
+    static constexpr int SCRATCH = (GA ? 4 * 9 * 2 * 32 : 9 * COUT * 32) * (int)sizeof(float);
+    static_assert(SCRATCH <= kWgStages * STAGE, "scratch fits the stages");
+    static constexpr size_t SMEM = (size_t)kWgStages * STAGE + 128;        // + alignment of the first stage
 };
 
-template <int CIN, int COUT>
-__global__ void __launch_bounds__(288)
-conv3x3_wgrad_kernel(const bf16* __restrict__ a, const bf16* __restrict__ gr, float* __restrict__ dw,
-                     float* __restrict__ db, int cin_real, int cout_real, int H, int W, int images) {
-    using C = WgradCfg<CIN, COUT>;
-    extern __shared__ __align__(16) bf16 sm[];
-    bf16* sA = sm;                                   // [CIN][PA]
-    bf16* sG = sm + CIN * C::PA;                     // [COUT][PG]
-    float* sDb = reinterpret_cast<float*>(sG + COUT * C::PG);
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;     // warp = tap
-    const int g = lane >> 2, t = lane & 3;
-    const int p = warp / 3, q = warp % 3;
-    constexpr int MT = COUT / 16, NT = CIN / 8;
-    float acc[MT][NT][4];
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[mt][nt][j] = 0.f;
-    for (int o = tid; o < COUT; o += 288) sDb[o] = 0.f;
+// instruction descriptor as idesc_m128, both operands MN-major
+__host__ __device__ constexpr uint32_t idesc_m128_mn(uint32_t n) { return idesc_m128(n) | (1u << 15) | (1u << 16); }
 
-    const int tx = W / kTile, ty = H / kTile;
-    const int tiles = tx * ty * images;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int im = tile / (tx * ty), rem = tile % (tx * ty);
-        const int r0 = (rem / tx) * kTile, c0 = (rem % tx) * kTile;
-        const size_t hw = (size_t)H * W;
-        __syncthreads();                             // previous tile's operands are consumed
-        // activation tile with halo, channel-major (8 channels of one plane per
-        // thread and pixel)
-        constexpr int NPA = C::HALO * C::HALO;
-        for (int e = tid; e < NPA * (CIN / 8); e += 288) {
-            const int pl = e / NPA, pix = e - pl * NPA, ch = pl * 8;
-            const int yy = pix / C::HALO, xx = pix % C::HALO;
-            const int gy = r0 + yy - 1, gx = c0 + xx - 1;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gy >= 0 && gy < H && gx >= 0 && gx < W)
-                v = *reinterpret_cast<const uint4*>(a + (((size_t)im * (CIN / 8) + pl) * hw + (size_t)gy * W + gx) * 8);
-            const bf16* vv = reinterpret_cast<const bf16*>(&v);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sA[(ch + j) * C::PA + pix] = vv[j];
+// floats of one CTA's partial vector of a layer (real channels)
+__host__ __device__ constexpr int wgrad_part(int cin, int cout) { return 9 * cin * cout + cout; }
+
+// ta, tg: TMA views of the activations [img][PA][H][W][8] and gradients
+// [img][PG][H][W][8] (see wgrad); part: gridDim.x partial vectors
+template <bool GA, int PA, int PG>
+__global__ void __launch_bounds__(128)
+conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tg,
+                 float* __restrict__ part, int cin, int cout, int H, int W, int images, int* __restrict__ err) {
+    using C = WgradCfg<GA, PA, PG>;
+    extern __shared__ unsigned char wg_raw[];
+    __shared__ __align__(8) unsigned long long full[kWgStages], empty[kWgStages], done;
+    __shared__ uint32_t tmem_base;
+    __shared__ float sDb[2][32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char* sm = wg_raw + ((128u - (sh_addr(wg_raw) & 127u)) & 127u);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sh_addr(&tmem_base)),
+                     "n"(C::TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int i = 0; i < kWgStages; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sh_addr(&full[i])) : "memory");
+            // a stage is free once its MMAs and both bias warps are done with it
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 3;" ::"r"(sh_addr(&empty[i])) : "memory");
         }
-        for (int e = tid; e < kTile * kTile * (COUT / 8); e += 288) {
-            const int pl = e / (kTile * kTile), pix = e - pl * (kTile * kTile), ch = pl * 8;
-            const int gy = r0 + pix / kTile, gx = c0 + pix % kTile;
-            const uint4 v =
-                *reinterpret_cast<const uint4*>(gr + (((size_t)im * (COUT / 8) + pl) * hw + (size_t)gy * W + gx) * 8);
-            const bf16* vv = reinterpret_cast<const bf16*>(&v);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sh_addr(&done)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    const int tiles_x = (W + kWgTW - 1) / kWgTW, per_img = tiles_x * ((H + kWgTH - 1) / kWgTH);
+    const int ntiles = per_img * images, G = gridDim.x;
+    bool ok = true;
+    int asked = 0;                                   // (producer) copies requested
+    float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (warp == 0 && lane == 0) {
+        int i = 0;
+        for (int t = blockIdx.x; t < ntiles; t += G, ++i) {
+            const int s = i % kWgStages;
+            if (i >= kWgStages && !mbar_wait_bounded(sh_addr(&empty[s]), (uint32_t)((i / kWgStages - 1) & 1))) {
+                ok = false;
+                break;
+            }
+            const int img = t / per_img, rem = t - img * per_img;
+            const int y0 = (rem / tiles_x) * kWgTH, x0 = (rem % tiles_x) * kWgTW;
+            const uint32_t bar = sh_addr(&full[s]), dst = sh_addr(sm + s * C::STAGE);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(C::ABYTES + C::GBYTES)
+                         : "memory");
+            // x in 4-byte elements, four per pixel and plane: 16-byte aligned; pixels
+            // outside the image read as zero
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                "%5}], [%6];" ::"r"(dst),
+                "l"(reinterpret_cast<uint64_t>(&ta)), "r"((x0 - 1) * 4), "r"(0), "r"(y0 - 1), "r"(img), "r"(bar)
+                : "memory");
+            asm volatile(
+                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                "%5}], [%6];" ::"r"(dst + C::ASTRIDE),
+                "l"(reinterpret_cast<uint64_t>(&tg)), "r"(x0 * 4), "r"(0), "r"(y0), "r"(img), "r"(bar)
+                : "memory");
+            asked = i + 1;
+        }
+        // every stage's last release has arrived before the CTA ends
+        for (int k = i > kWgStages ? i - kWgStages : 0; ok && k < i; ++k)
+            ok = mbar_wait_bounded(sh_addr(&empty[k % kWgStages]), (uint32_t)((k / kWgStages) & 1));
+    } else if (warp == 1 && lane == 0) {
+        int i = 0;
+        for (int t = blockIdx.x; t < ntiles; t += G, ++i) {
+            const int s = i % kWgStages;
+            if (!mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((i / kWgStages) & 1))) {
+                ok = false;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t aB = sh_addr(sm + s * C::STAGE), gB = aB + C::ASTRIDE;
+#pragma unroll 1
+            for (int r = 0; r < kWgTH; r += C::STEP) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) sG[(ch + j) * C::PG + pix] = vv[j];
+                for (int kc = 0; kc < kWgTW / 16; ++kc) {
+                    const uint32_t gAddr = gB + (uint32_t)(r * PG * kWgTW + 16 * kc) * 16;
+                    const uint64_t gd = umma_desc(gAddr, 128, kWgTW * 16);
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const uint64_t ad = umma_desc(aB + (uint32_t)(r * PA * C::AW + 16 * kc + dx) * 16, 128,
+                                                      C::AW * 16);
+                        umma_f16(tmem + (uint32_t)(C::N * dx), GA ? gd : ad, GA ? ad : gd, idesc_m128_mn(C::N),
+                                 (i | r | kc) != 0 ? 1u : 0u);
+                    }
+                }
+            }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             sh_addr(&empty[s]))
+                         : "memory");
+        }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sh_addr(&done))
+                     : "memory");
+    } else if (warp >= 2) {
+        // bias: thread j of the 64 sums plane j % PG over every (64 / PG)-th pixel
+        const int j = tid - 64, pl = j % PG;
+        int i = 0;
+        for (int t = blockIdx.x; t < ntiles; t += G, ++i) {
+            const int s = i % kWgStages;
+            if (!mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((i / kWgStages) & 1))) {
+                ok = false;
+                break;
+            }
+            const uint4* g4 = reinterpret_cast<const uint4*>(sm + s * C::STAGE + C::ASTRIDE);
+#pragma unroll 4
+            for (int px = j / PG; px < kWgTW * kWgTH; px += 64 / PG) {
+                const uint4 v = g4[((px / kWgTW) * PG + pl) * kWgTW + px % kWgTW];
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    db[2 * h] += __uint_as_float(w[h] << 16);
+                    db[2 * h + 1] += __uint_as_float(w[h] & 0xFFFF0000u);
+                }
+            }
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sh_addr(&empty[s])) : "memory");
+        }
+    }
+    __syncwarp();
+    ok = __syncthreads_and(ok) != 0;
+    // the accumulators are complete (and, on a failure, every MMA issued is:
+    // the commit above tracks all of them)
+    ok = __syncthreads_and(mbar_wait_bounded(sh_addr(&done), 0u) && ok) != 0;
+    if (!ok) {
+        // a wait ran out: let the copies still in flight land (bounded) before leaving
+        if (tid == 0) {
+            atomicExch(err, 1);
+            for (int i = asked > kWgStages ? asked - kWgStages : 0; i < asked; ++i)
+                mbar_wait_bounded(sh_addr(&full[i % kWgStages]), (uint32_t)((i / kWgStages) & 1));
+        }
+    } else {
+        tc_fence_after();
+        float* __restrict__ mine = part + (size_t)blockIdx.x * wgrad_part(cin, cout);
+        float* scr = reinterpret_cast<float*>(sm);
+        const uint32_t tw = tmem + ((uint32_t)(32 * warp) << 16);
+        if (warp >= 2) {
+            // lanes with the same plane add up: 32 / PG lanes per plane
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+#pragma unroll
+                for (int o = 16; o >= PG; o >>= 1) db[e] += __shfl_down_sync(0xffffffffu, db[e], o);
+                if (lane < PG) sDb[warp - 2][8 * lane + e] = db[e];
+            }
+        }
+        if constexpr (!GA) {
+            // lane = input channel, warp = activation row ay; columns: gradient row gy, output channel
+            constexpr int CO = C::COUT;
+            for (int gy = 0; gy < 2; ++gy) {
+                const int dy = warp - gy;
+                if (gy == 1) __syncthreads();        // the rows of gy = 0 are in the scratch
+                if (dy < 0 || dy > 2) continue;
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                    for (int q = 0; q < CO; q += CO < 16 ? 8 : 16) {
+                        constexpr int NV = CO < 16 ? 8 : 16;
+                        float v[NV];
+                        tmem_ld(tw + (uint32_t)(C::N * dx + CO * gy + q), v);
+#pragma unroll
+                        for (int c = 0; c < NV; ++c) {
+                            const int tap = 3 * dy + dx;
+                            float* sp = scr + (tap * CO + q + c) * 32 + lane;
+                            if (gy == 0) *sp = v[c];
+                            // (the rows of gy = 0 cover every dy, so each entry is complete here)
+                            else if (q + c < cout) mine[(tap * cout + q + c) * 32 + lane] = *sp + v[c];
+                        }
+                    }
+                }
+            }
+        } else {
+            // lane = output channel, warp = gradient row gy; columns: activation row ay = gy + dy, input channel
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    float v[8];
+                    tmem_ld(tw + (uint32_t)(C::N * dx + 8 * (warp + dy)), v);
+                    scr[((warp * 9 + 3 * dy + dx) * 2 + 0) * 32 + lane] = v[0];
+                    scr[((warp * 9 + 3 * dy + dx) * 2 + 1) * 32 + lane] = v[1];
+                }
+            }
+            __syncthreads();
+            for (int e = tid; e < 9 * 2 * 32; e += 128) {
+                const int co = e & 31, ci = (e >> 5) & 1, tap = e >> 6;
+                float v = 0.f;
+#pragma unroll
+                for (int gy = 0; gy < 4; ++gy) v += scr[((gy * 9 + tap) * 2 + ci) * 32 + co];
+                mine[(tap * 32 + co) * 2 + ci] = v;
+            }
         }
         __syncthreads();
-        // bias gradient: channel o = tid % 32 sums every 9th pixel row
-        if ((tid & 31) < COUT) {
-            const int o = tid & 31;
-            float s = 0.f;
-            for (int px = warp; px < kTile * kTile; px += 9) s += __bfloat162float(sG[o * C::PG + px]);
-            atomicAdd(sDb + o, s);
-        }
-        // K loop: one output row of 16 pixels per step
-#pragma unroll 2
-        for (int rr = 0; rr < kTile; ++rr) {
-            uint32_t af[MT][4];
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt) {
-                // A[m][k] = G[pixel k][channel m]
-                const bf16* gp = sG + (mt * 16 + g) * C::PG + rr * kTile + 2 * t;
-                af[mt][0] = ld32(gp);
-                af[mt][1] = ld32(gp + 8 * C::PG);
-                af[mt][2] = ld32(gp + 8);
-                af[mt][3] = ld32(gp + 8 * C::PG + 8);
-            }
-            const int base = (rr + p) * C::HALO + q + 2 * t;  // pixel (rr + p - 1, 2t + q - 1) + halo
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                // B[k][n] = A_tap[pixel k][channel n]: two pixels of one channel
-                const bf16* ap = sA + (nt * 8 + g) * C::PA + base;
-                const uint32_t b0 = pack2(ap[0], ap[1]);
-                const uint32_t b1 = pack2(ap[8], ap[9]);
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) mma_bf16(acc[mt][nt], af[mt][0], af[mt][1], af[mt][2], af[mt][3], b0, b1);
-            }
-        }
+        if (tid < cout) mine[9 * cin * cout + tid] = sDb[0][tid] + sDb[1][tid];
     }
-    // C[m][n] = dW[o = m][i = n] of this tap
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int o = mt * 16 + g + (j >= 2 ? 8 : 0);
-                const int i = nt * 8 + 2 * t + (j & 1);
-                if (o < cout_real && i < cin_real) atomicAdd(dw + ((size_t)o * cin_real + i) * 9 + warp, acc[mt][nt][j]);
-            }
-        }
-    }
+    tc_fence_before();
     __syncthreads();
-    for (int o = tid; o < cout_real; o += 288) atomicAdd(db + o, sDb[o]);
+    tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(C::TMEM_COLS) : "memory");
+}
+
+// The layers' gradients from the CTAs' partial vectors (ncta per layer, added
+// in a fixed order). Block: 32 entries of one partial vector x 8 shares of the
+// CTAs. ws: per layer ncta x wgrad_part floats, at ncta * base.
+struct ReduceArgs {
+    int cin[kLayers], cout[kLayers], block0[kLayers + 1];
+    long long base[kLayers], param[kLayers];
+};
+__global__ void __launch_bounds__(256)
+wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ grads, int ncta, ReduceArgs a) {
+    __shared__ float red[8][33];
+    int l = 0;
+    while (l + 1 < kLayers && (int)blockIdx.x >= a.block0[l + 1]) ++l;
+    const int cin = a.cin[l], cout = a.cout[l], n = wgrad_part(cin, cout);
+    const int lane = threadIdx.x & 31, sh = threadIdx.x >> 5;
+    const int e = ((int)blockIdx.x - a.block0[l]) * 32 + lane;
+    float v = 0.f;
+    if (e < n) {
+        const float* p = ws + a.base[l] * ncta + e;
+#pragma unroll 4
+        for (int c = sh; c < ncta; c += 8) v += p[(size_t)c * n];
+    }
+    red[sh][lane] = v;
+    __syncthreads();
+    if (sh == 0 && e < n) {
+        v = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v += red[k][lane];
+        const int nw = 9 * cin * cout;
+        // partial [tap][cout][cin] -> parameters w[cout][cin][3][3], then the bias
+        int o = e;
+        if (e < nw) {
+            const int tap = e / (cin * cout), co = (e / cin) % cout, ci = e % cin;
+            o = (co * cin + ci) * 9 + tap;
+        }
+        grads[a.param[l] + o] = v;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -739,13 +920,32 @@ cudaError_t conv_tc(const bf16* in, const bf16* w, const float* bias, void* out,
     return cudaGetLastError();
 }
 
-template <int CIN, int COUT>
-cudaError_t wgrad(const bf16* a, const bf16* g, float* dw, float* db, int cin_real, int cout_real, int count,
-                  int H, int W, int sms, cudaStream_t s) {
-    const int tiles = (H / kTile) * (W / kTile) * count;
-    const int grid = std::min(tiles, 2 * sms);
-    conv3x3_wgrad_kernel<CIN, COUT><<<grid, 288, WgradCfg<CIN, COUT>::SMEM, s>>>(a, g, dw, db, cin_real, cout_real, H,
-                                                                                  W, count);
+// One layer's weight and bias gradients into the CTAs' partial vectors. The
+// planes are viewed by TMA as 4-D tensors (4 W four-byte elements of a plane
+// row, planes, H, images), so that a tile lands as [row][plane][column][8].
+template <bool GA, int PA, int PG>
+cudaError_t wgrad(const bf16* a, const bf16* g, float* part, int cin, int cout, int count, int H, int W, int grid,
+                  int* err, cudaStream_t s) {
+    using C = WgradCfg<GA, PA, PG>;
+    cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc<GA, PA, PG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)C::SMEM);
+    if (e != cudaSuccess) return e;
+    const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+    if (!enc) return cudaErrorNotSupported;
+    CUtensorMap tm[2];
+    for (int k = 0; k < 2; ++k) {
+        const cuuint64_t np = k == 0 ? PA : PG, plane = (cuuint64_t)W * H * 16;
+        const cuuint64_t dims[4] = {(cuuint64_t)W * 4, np, (cuuint64_t)H, (cuuint64_t)count};
+        const cuuint64_t strides[3] = {plane, (cuuint64_t)W * 16, plane * np};
+        const cuuint32_t box[4] = {(cuuint32_t)(k == 0 ? C::AW : kWgTW) * 4, (cuuint32_t)np,
+                                   (cuuint32_t)(k == 0 ? C::AR : kWgTH), 1};
+        const cuuint32_t es[4] = {1, 1, 1, 1};
+        if (enc(&tm[k], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, const_cast<bf16*>(k == 0 ? a : g), dims, strides, box, es,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+    }
+    conv3x3_wgrad_tc<GA, PA, PG><<<grid, 128, C::SMEM, s>>>(tm[0], tm[1], part, cin, cout, H, W, count, err);
     ++g_cnn_launches;
     return cudaGetLastError();
 }
@@ -769,6 +969,7 @@ struct admm_cnn_s {
     float* out = nullptr;          // output, 4 channels FP32
     bf16* gbuf[2] = {};            // gradient ping-pong, 32 channels
     bf16* gout = nullptr;          // output gradient, 16 channels
+    float* wpart = nullptr;        // weight-gradient partial vectors, one per CTA and layer
     double* loss = nullptr;        // device accumulator
     double* h_loss = nullptr;      // pinned
     int* tc_err = nullptr;         // set by a tensor-core convolution whose bounded wait ran out
@@ -840,27 +1041,41 @@ int forward(admm_cnn_s* n, int count, int H, int W, const float* ybar, const uin
     return run_layers(n, count, H, W, keep, s);
 }
 
-// loss, gradients into n->grads (zeroed first)
+// loss, gradients into n->grads
 int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const float* chan_w, cudaStream_t s) {
     const long long npx = (long long)count * H * W;
     CKC(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
-    CKC(cudaMemsetAsync(n->grads, 0, param_count() * sizeof(float), s));
     const float4 cw = make_float4(chan_w[0], chan_w[1], chan_w[2], chan_w[3]);
     cnn_loss_kernel<<<(unsigned)((npx + 255) / 256), 256, 0, s>>>(n->out, target, cw, n->gout, n->loss, npx,
                                                                    (long long)H * W);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
+    const int tiles = ((H + kWgTH - 1) / kWgTH) * ((W + kWgTW - 1) / kWgTW) * count;
+    const int ncta = std::min(tiles, n->sms);
+    ReduceArgs ra{};
+    long long base = 0;
+    int blocks = 0;
+    for (int l = 0; l < kLayers; ++l) {
+        const int np = wgrad_part(layer_cin(l), layer_cout(l));
+        ra.cin[l] = layer_cin(l);
+        ra.cout[l] = layer_cout(l);
+        ra.base[l] = base;
+        ra.param[l] = param_offset(l);
+        ra.block0[l] = blocks;
+        base += np;
+        blocks += (np + 31) / 32;
+    }
+    ra.block0[kLayers] = blocks;
     const bf16* g = n->gout;                        // gradient in the output of layer l
     for (int l = kLayers - 1; l >= 0; --l) {
-        float* dw = n->grads + param_offset(l);
-        float* db = dw + (long long)layer_cout(l) * layer_cin(l) * 9;
+        float* pt = n->wpart + ra.base[l] * ncta;
         const bf16* a_in = l == 0 ? n->a0 : n->act[l - 1];
         if (l == kLayers - 1)
-            CKC((wgrad<32, 16>(a_in, g, dw, db, kWidth, kOut, count, H, W, n->sms, s)));
+            CKC((wgrad<false, 4, 2>(a_in, g, pt, kWidth, kOut, count, H, W, ncta, n->tc_err, s)));
         else if (l == 0)
-            CKC((wgrad<8, 32>(a_in, g, dw, db, kIn, kWidth, count, H, W, n->sms, s)));
+            CKC((wgrad<true, 1, 4>(a_in, g, pt, kIn, kWidth, count, H, W, ncta, n->tc_err, s)));
         else
-            CKC((wgrad<32, 32>(a_in, g, dw, db, kWidth, kWidth, count, H, W, n->sms, s)));
+            CKC((wgrad<false, 4, 4>(a_in, g, pt, kWidth, kWidth, count, H, W, ncta, n->tc_err, s)));
         if (l == 0) break;
         bf16* gnext = n->gbuf[l & 1];
         if (l == kLayers - 1)
@@ -869,6 +1084,9 @@ int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const 
             CKC((conv_tc<32, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
         g = gnext;
     }
+    wgrad_reduce_kernel<<<blocks, 256, 0, s>>>(n->wpart, n->grads, ncta, ra);
+    ++g_cnn_launches;
+    CKC(cudaGetLastError());
     return ADMM_OK;
 }
 
@@ -920,7 +1138,8 @@ int admm_cnn_create(admm_cnn_t* out, long long max_pixels, int training) {
     if (n->training) {
         if ((rc = dalloc(n, &n->grads, P)) || (rc = dalloc(n, &n->m, P)) || (rc = dalloc(n, &n->v, P)) ||
             (rc = dalloc(n, &n->gbuf[0], px * kWidth)) || (rc = dalloc(n, &n->gbuf[1], px * kWidth)) ||
-            (rc = dalloc(n, &n->gout, px * 16)) || (rc = dalloc(n, &n->loss, 1)))
+            (rc = dalloc(n, &n->gout, px * 16)) || (rc = dalloc(n, &n->loss, 1)) ||
+            (rc = dalloc(n, &n->wpart, (size_t)P * n->sms)))
             return bail(rc);
         if (admm::alloc_fault_fire() || cudaHostAlloc(&n->h_loss, sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
             n->h_loss = nullptr;
