@@ -14,8 +14,9 @@
 // the MMA consumes them.
 //
 // Every convolution of the forward pass and every input gradient runs on
-// tcgen05 (conv3x3_tc below): the 32-channel layers with bias and ReLU, the
-// input gradients gated by the ReLU of the layer below, and the last layer
+// tcgen05 (conv3x3_rows, and conv3x3_tc for the first layer and for widths that
+// strips of 128 columns do not fit): the 32-channel layers with bias and ReLU,
+// the input gradients gated by the ReLU of the layer below, and the last layer
 // (4 outputs padded to 16) with bias into FP32.
 //
 // The weight gradients are contractions over pixels, also on tcgen05
@@ -226,6 +227,24 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// clear N (16 or 32) consecutive columns of this warp's accumulator lanes
+template <int N>
+__device__ __forceinline__ void tmem_zero(uint32_t taddr) {
+    static_assert(N == 16 || N == 32, "columns");
+    if constexpr (N == 32)
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,"
+            "%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n\ttcgen05.wait::st.sync.aligned;\n" ::"r"(taddr),
+            "r"(0u)
+            : "memory");
+    else
+        asm volatile(
+            "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};\n\t"
+            "tcgen05.wait::st.sync.aligned;\n" ::"r"(taddr),
+            "r"(0u)
+            : "memory");
+}
+
 constexpr int kTcTW = 8, kTcTH = 16;                 // output tile (M = 128)
 constexpr int kTcHW = kTcTW + 2, kTcHH = kTcTH + 2;  // halo tile
 constexpr int kTcNP = kTcHW * kTcHH;                 // 180 halo pixels
@@ -432,6 +451,294 @@ conv3x3_tc(const __grid_constant__ CUtensorMap tin, const bf16* __restrict__ wpk
     tc_fence_after();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// 3 x 3 convolution of 16 or 32 input channels, streaming down the image
+//
+// A CTA walks rows of a strip of 128 columns (M = 128, accumulator row =
+// column). An input row is the A operand of three output rows at once: the
+// accumulators of output rows r - 1, r, r + 1 are three slots of COUT columns
+// in tensor memory (slot = row mod 3), and one MMA of N = 3 COUT adds input row
+// r's products with the weights of dy = 2, 1, 0 to them. The weight blocks lie
+// in the cyclic order dy = 2 1 0 2 1, so each of the three rotations of the
+// slots is a window of three consecutive blocks. That is 6 MMAs (dx, half of
+// the channels) per row of 128 pixels and 7 KB of shared-memory operand reads
+// each, 2.6 cycles per pixel and SM where one 128 x 32 MMA per tap reads 5.6
+// (conv3x3_tc): the layer is then bound by its HBM traffic (64 B in and out per
+// pixel, 5.6 cycles), with no column halo in it and two halo rows per segment.
+// Every output sees its products in the order (dy, dx, channels) of
+// conv3x3_tc, so the results have the same bits.
+//
+// Work: the count x strips x H strip rows are cut into equal ranges, one per
+// CTA (three CTAs per SM), each a segment or two of consecutive rows of one
+// strip. Warp 0 copies input rows (cp.async.bulk, one per plane of eight
+// channels) kRowStages ahead and writes the zeros outside the image; lane 0 of
+// warp 1 issues the MMAs; warps 2..5 read a finished accumulator, clear its
+// slot for the row that takes it over, and store the row: bias + ReLU or the
+// ReLU gate of the layer below into BF16 planes, or bias into FP32 outputs.
+// While a CTA's MMAs wait for a slot to be read, the other CTAs' run.
+// Hidden layer at 16 x 512^2: 103 us (5.2 TB/s of activations), 126 us as
+// 8 x 16 tiles; the last layer 72 against 95 us.
+// ---------------------------------------------------------------------------
+constexpr int kStrip = 128, kRowPx = kStrip + 2, kRowStages = 4;
+
+template <int CIN, int MODE>
+struct RowsCfg {
+    static constexpr int CH = CIN / 8, COUT = MODE == kModeOutF32 ? 16 : 32;
+    static constexpr int STAGE = (CH * kRowPx * 16 + 127) / 128 * 128;   // one input row with its two halo columns
+    static constexpr int WBLK = 2 * 5 * COUT * 16;                       // weights of one (dx, channel half): 5 blocks
+    static constexpr int NWB = 3 * (CIN / 16);
+    static constexpr int N = 3 * COUT;
+    static constexpr int TMEM_COLS = N <= 64 ? 64 : 128;
+    static constexpr size_t SMEM = (size_t)kRowStages * STAGE + (size_t)NWB * WBLK + 128;
+    static constexpr int CTAS = 3;                                       // per SM
+};
+
+template <int CIN, int MODE>
+__global__ void __launch_bounds__(192, 3)
+conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const float* __restrict__ bias,
+             void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, int* __restrict__ err) {
+    using C = RowsCfg<CIN, MODE>;
+    constexpr int CH = C::CH, COUT = C::COUT, S = kRowStages;
+    extern __shared__ unsigned char rows_raw[];
+    __shared__ __align__(8) unsigned long long full[S], empty[S], acc_full[3], acc_empty[3], done;
+    __shared__ __align__(16) float smB[32];
+    __shared__ uint32_t tmem_base;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    unsigned char* sm = rows_raw + ((128u - (sh_addr(rows_raw) & 127u)) & 127u);
+    unsigned char* smW = sm + S * C::STAGE;
+    // weights [dx][channel half][8-channel chunk][block, output channel][8]
+    for (int e = tid; e < C::NWB * 2 * 5 * COUT; e += 192) {
+        const int n = e % (5 * COUT), kh = (e / (5 * COUT)) % 2, blk = e / (10 * COUT);
+        const int dx = blk / (CIN / 16), j = blk % (CIN / 16), co = n % COUT;
+        const int dy = (5 - n / COUT) % 3;            // blocks 0..4: 2 1 0 2 1
+        cp_async16(smW + (size_t)e * 16, wpk + ((size_t)(dy * 3 + dx) * COUT + co) * CIN + (2 * j + kh) * 8);
+    }
+    if (MODE != kModeGateBf16 && tid < (MODE == kModeOutF32 ? kOut : COUT)) smB[tid] = bias[tid];
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sh_addr(&tmem_base)),
+                     "n"(C::TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    auto bar_init = [](unsigned long long* b, uint32_t n) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sh_addr(b)), "r"(n) : "memory");
+    };
+    auto arrive = [](unsigned long long* b) {
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sh_addr(b)) : "memory");
+    };
+    auto commit = [](unsigned long long* b) {
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sh_addr(b))
+                     : "memory");
+    };
+    if (tid == 0) {
+        for (int i = 0; i < S; ++i) {
+            bar_init(&full[i], 1);
+            bar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 3; ++i) {
+            bar_init(&acc_full[i], 1);
+            bar_init(&acc_empty[i], 4);
+        }
+        bar_init(&done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    cp_async_wait_all();
+    fence_async_shared();        // the weights (generic proxy) are visible to the tensor cores
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base;
+    const int strips = (W + kStrip - 1) / kStrip;
+    const long long total = (long long)count * strips * H;
+    const long long a0 = total * blockIdx.x / gridDim.x, a1 = total * (blockIdx.x + 1) / gridDim.x;
+    const size_t hw = (size_t)H * W;
+    bool ok = true;
+    int asked = 0, used = 0;     // input rows requested; released by the MMAs (producer)
+    if (warp == 0) {
+        int n = 0;
+        for (long long pos = a0; pos < a1 && ok;) {
+            const int col = (int)(pos / H), y0 = (int)(pos - (long long)col * H);
+            const int R = (int)min((long long)(H - y0), a1 - pos);
+            const int img = col / strips, xs = (col - img * strips) * kStrip;
+            pos += R;
+            const int c0 = max(xs - 1, 0), c1 = min(xs + kStrip + 1, W);
+            const int lo = c0 - (xs - 1), hi = c1 - (xs - 1);          // slots [lo, hi) hold image columns
+            for (int i = 0; i < R + 2; ++i, ++n) {
+                const int s = n % S, r = y0 - 1 + i;
+                if (n >= S) {
+                    ok = mbar_wait_bounded(sh_addr(&empty[s]), (uint32_t)((n / S - 1) & 1));
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    used = n - S + 1;
+                }
+                unsigned char* st = sm + s * C::STAGE;
+                const bool inside = r >= 0 && r < H;
+                const int h0 = inside ? lo : kRowPx, nz = kRowPx - (inside ? hi - lo : 0);
+                if (nz > 0) {
+                    // zeros outside the image: slots [0, h0) and, for a row inside, [hi, kRowPx)
+                    for (int e = lane; e < nz * CH; e += 32) {
+                        const int pl = e / nz, k = e - pl * nz;
+                        const int slot = k < h0 ? k : hi + (k - h0);
+                        *reinterpret_cast<uint4*>(st + (pl * kRowPx + slot) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    }
+                    fence_async_shared();
+                    __syncwarp();
+                }
+                if (lane == 0) {
+                    const uint32_t bar = sh_addr(&full[s]);
+                    if (inside) {
+                        const uint32_t bytes = (uint32_t)(hi - lo) * 16u;
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes * CH)
+                                     : "memory");
+                        const bf16* src = in + ((size_t)img * CH * hw + (size_t)r * W + c0) * 8;
+                        for (int pl = 0; pl < CH; ++pl)
+                            asm volatile(
+                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                    sh_addr(st + (pl * kRowPx + lo) * 16)),
+                                "l"(src + (size_t)pl * hw * 8), "r"(bytes), "r"(bar)
+                                : "memory");
+                    } else {
+                        arrive(&full[s]);
+                    }
+                }
+                asked = n + 1;
+            }
+        }
+        // every stage's last release has arrived before the CTA ends
+        for (int k = max(0, n - S); ok && k < n; ++k)
+            ok = mbar_wait_bounded(sh_addr(&empty[k % S]), (uint32_t)((k / S) & 1));
+    } else if (warp == 1 && lane == 0) {
+        int n = 0;
+        uint32_t eph = 0, need = 7;                  // slots whose clearing is not yet seen (at first: all)
+        const uint32_t wB = sh_addr(smW);
+        auto slot_clear = [&](int k) -> bool {
+            if (!((need >> k) & 1u)) return true;
+            if (!mbar_wait_bounded(sh_addr(&acc_empty[k]), (eph >> k) & 1u)) return false;
+            eph ^= 1u << k;
+            need &= ~(1u << k);
+            return true;
+        };
+        for (long long pos = a0; pos < a1 && ok;) {
+            const int y0 = (int)(pos % H);
+            const int R = (int)min((long long)(H - y0), a1 - pos);
+            pos += R;
+            for (int i = 0; i < R + 2; ++i, ++n) {
+                const int s = n % S, ph = n % 3;
+                // (first row of a segment: all three slots)
+                ok = mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((n / S) & 1)) && slot_clear((ph + 1) % 3) &&
+                     (i > 0 || (slot_clear(ph) && slot_clear((ph + 2) % 3)));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t aB = sh_addr(sm + s * C::STAGE);
+                const uint32_t w0 = wB + (uint32_t)((4 - ph) % 3) * (COUT * 16);   // window start: 1, 0, 2
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                    for (int j = 0; j < CIN / 16; ++j) {
+                        const uint64_t a = umma_desc(aB + (2 * j * kRowPx + dx) * 16, kRowPx * 16, 128);
+                        const uint64_t b = umma_desc(w0 + (dx * (CIN / 16) + j) * C::WBLK, 5 * COUT * 16, 128);
+                        umma_f16(tmem, a, b, idesc_m128(C::N), 1u);
+                    }
+                }
+                commit(&empty[s]);
+                commit(&acc_full[(ph + 2) % 3]);     // output row r - 1 is complete
+                need |= 1u << ((ph + 2) % 3);
+            }
+            if (!ok) break;
+            // the two rows that the segment's last input row has begun are dropped
+            commit(&acc_full[(n - 1) % 3]);
+            commit(&acc_full[n % 3]);
+            need = 7;
+        }
+        commit(&done);
+    } else if (warp >= 2) {
+        const int q = warp & 3;                      // this warp's quarter of the tensor-memory lanes
+        const uint32_t tw = tmem + ((uint32_t)(32 * q) << 16);
+        // clear slot k and hand it to the MMAs
+        auto release = [&](int k) {
+            tmem_zero<COUT>(tw + (uint32_t)(COUT * k));
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive(&acc_empty[k]);
+        };
+        for (int k = 0; k < 3; ++k) release(k);
+        int n0 = 0;
+        uint32_t fph = 0;
+        for (long long pos = a0; pos < a1 && ok;) {
+            const int col = (int)(pos / H), y0 = (int)(pos - (long long)col * H);
+            const int R = (int)min((long long)(H - y0), a1 - pos);
+            const int img = col / strips, xs = (col - img * strips) * kStrip;
+            pos += R;
+            const int c = xs + 32 * q + lane;
+            for (int d = 0; d < R + 4; ++d) {
+                const int k = (n0 + d + 2) % 3, o = y0 - 2 + d;
+                const bool keep = d >= 2 && d < R + 2 && c < W;
+                // pixel's slot in plane 0 of its image; plane p is p hw slots further
+                const size_t px = (size_t)img * (MODE == kModeOutF32 ? 1 : 4) * hw + (size_t)o * W + c;
+                uint4 gv[4];
+                if constexpr (MODE == kModeGateBf16) {
+                    const uint4* gp = reinterpret_cast<const uint4*>(gate) + px;
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) gv[p] = keep ? __ldcs(gp + p * hw) : make_uint4(0u, 0u, 0u, 0u);
+                }
+                ok = __all_sync(0xffffffffu, mbar_wait_bounded(sh_addr(&acc_full[k]), (fph >> k) & 1u));
+                if (!ok) break;
+                fph ^= 1u << k;
+                tc_fence_after();
+                float v[COUT];
+                if constexpr (COUT == 32) tmem_ld32(tw + (uint32_t)(COUT * k), v);
+                else tmem_ld(tw + (uint32_t)(COUT * k), v);
+                release(k);
+                if (!keep) continue;
+                if constexpr (MODE == kModeOutF32) {
+                    reinterpret_cast<float4*>(out)[px] =
+                        make_float4(v[0] + smB[0], v[1] + smB[1], v[2] + smB[2], v[3] + smB[3]);
+                } else {
+                    uint4* op = reinterpret_cast<uint4*>(out) + px;
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        uint32_t pk[4];
+                        if constexpr (MODE == kModeReluBf16) {
+                            const float4 b0 = *reinterpret_cast<const float4*>(smB + 8 * p);
+                            const float4 b1 = *reinterpret_cast<const float4*>(smB + 8 * p + 4);
+                            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+                            for (int h = 0; h < 4; ++h)
+                                pk[h] = pack2(__float2bfloat16(fmaxf(v[8 * p + 2 * h] + b[2 * h], 0.f)),
+                                              __float2bfloat16(fmaxf(v[8 * p + 2 * h + 1] + b[2 * h + 1], 0.f)));
+                        } else {
+                            const uint32_t gw[4] = {gv[p].x, gv[p].y, gv[p].z, gv[p].w};
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                const float g0 = __uint_as_float(gw[h] << 16), g1 = __uint_as_float(gw[h] & 0xFFFF0000u);
+                                pk[h] = pack2(__float2bfloat16(g0 > 0.f ? v[8 * p + 2 * h] : 0.f),
+                                              __float2bfloat16(g1 > 0.f ? v[8 * p + 2 * h + 1] : 0.f));
+                            }
+                        }
+                        op[p * hw] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    }
+                }
+            }
+            n0 += R + 2;
+        }
+    }
+    __syncwarp();
+    ok = __syncthreads_and(ok) != 0;
+    // every MMA issued is complete
+    ok = __syncthreads_and(mbar_wait_bounded(sh_addr(&done), 0u) && ok) != 0;
+    if (!ok && tid == 0) {
+        // a wait ran out: let the copies still in flight land (bounded) before leaving
+        atomicExch(err, 1);
+        for (int k = max(used, asked - S); k < asked; ++k)
+            mbar_wait_bounded(sh_addr(&full[k % S]), (uint32_t)((k / S) & 1));
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(C::TMEM_COLS) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -920,6 +1227,34 @@ cudaError_t conv_tc(const bf16* in, const bf16* w, const float* bias, void* out,
     return cudaGetLastError();
 }
 
+// Strips of 128 columns against 8 x 16 tiles: a strip costs the same however
+// much of it lies in the image, and the tiles take 1.23 times the strips' time
+// on full strips (103 / 126 us per hidden layer at 16 x 512^2), so the strips
+// are taken while they are at most a quarter wider than the image.
+bool rows_fit(int W) { return ((W + kStrip - 1) / kStrip) * kStrip * 4 <= W * 5; }
+
+// One layer of 16 or 32 input channels: conv3x3_rows where its strips of 128
+// columns fit the width, else the 8 x 16 tiles of conv3x3_tc
+template <int CIN, int MODE>
+cudaError_t conv_rows(const bf16* in, const bf16* w, const float* bias, void* out, const bf16* gate, int count, int H,
+                      int W, int sms, int* err, cudaStream_t s) {
+    using C = RowsCfg<CIN, MODE>;
+    const int strips = (W + kStrip - 1) / kStrip;
+    if (!rows_fit(W)) return conv_tc<CIN, MODE>(in, w, bias, out, gate, count, H, W, sms, err, s);
+    cudaError_t e = cudaFuncSetAttribute(conv3x3_rows<CIN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)C::SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(conv3x3_rows<CIN, MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+    // (at least eight strip rows per CTA: each segment adds two halo rows)
+    const long long total = (long long)count * strips * H;
+    const int grid = (int)std::max(1LL, std::min((long long)C::CTAS * sms, total / 8));
+    conv3x3_rows<CIN, MODE><<<grid, 192, C::SMEM, s>>>(in, w, bias, out, gate, H, W, count, err);
+    ++g_cnn_launches;
+    return cudaGetLastError();
+}
+
 // One layer's weight and bias gradients into the CTAs' partial vectors. The
 // planes are viewed by TMA as 4-D tensors (4 W four-byte elements of a plane
 // row, planes, H, images), so that a tile lands as [row][plane][column][8].
@@ -1018,13 +1353,13 @@ int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, cudaStream_t s
     for (int l = 0; l < kLayers; ++l) {
         const float* b = n->params + param_offset(l) + (long long)layer_cout(l) * layer_cin(l) * 9;
         if (l == kLayers - 1) {
-            CKC((conv_tc<32, kModeOutF32>(cur, n->wf[l], b, n->out, nullptr, count, H, W, n->sms, n->tc_err, s)));
+            CKC((conv_rows<32, kModeOutF32>(cur, n->wf[l], b, n->out, nullptr, count, H, W, n->sms, n->tc_err, s)));
         } else {
             bf16* dst = keep ? n->act[l] : n->act[l & 1];
             if (l == 0)
                 CKC((conv_tc<8, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
             else
-                CKC((conv_tc<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
+                CKC((conv_rows<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
             cur = dst;
         }
     }
@@ -1079,9 +1414,9 @@ int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const 
         if (l == 0) break;
         bf16* gnext = n->gbuf[l & 1];
         if (l == kLayers - 1)
-            CKC((conv_tc<16, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
+            CKC((conv_rows<16, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
         else
-            CKC((conv_tc<32, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
+            CKC((conv_rows<32, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
         g = gnext;
     }
     wgrad_reduce_kernel<<<blocks, 256, 0, s>>>(n->wpart, n->grads, ncta, ra);
