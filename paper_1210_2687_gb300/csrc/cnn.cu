@@ -103,7 +103,25 @@ __global__ void cnn_input_kernel(const float* __restrict__ ybar, const uint8_t* 
         make_uint4(pack2(__float2bfloat16(y), __float2bfloat16(obs ? 1.f : 0.f)), 0u, 0u, 0u);
 }
 
-enum { kModeReluBf16 = 0, kModeOutF32 = 1, kModeGateBf16 = 2 };   // epilogues of conv3x3_tc
+// epilogues of the convolutions
+enum { kModeReluBf16 = 0, kModeOutF32 = 1, kModeGateBf16 = 2, kModeStart = 3 };
+
+// planes of eight channels that a convolution's input has in memory: the output
+// gradient's 4 channels are one plane, the second of its 16-channel operand zeros
+__host__ __device__ constexpr int stored_planes(int cin) { return cin == 16 ? 1 : cin / 8; }
+
+// Where the last layer writes a predicted start (kModeStart): x0 = s0 o0, d1 =
+// s1 o1, d2 = (s2 o2, s2 o3) of image i to x0 + i hw and d0 + 3 i hw or, for
+// separately stored problems (a batch solve's learned start), px0[i], pd0[i]
+constexpr int kWsBatch = 16;
+struct StartOut {
+    float s0, s1, s2;
+    int separate;
+    float* x0;
+    float* d0;
+    float* px0[kWsBatch];
+    float* pd0[kWsBatch];
+};
 
 // ---------------------------------------------------------------------------
 // 3 x 3 convolution on the fifth-generation tensor cores (tcgen05.mma,
@@ -501,7 +519,8 @@ constexpr int kStrip = 128, kRowPx = kStrip + 2, kRowStages = 4;
 
 template <int CIN, int MODE>
 struct RowsCfg {
-    static constexpr int CH = CIN / 8, COUT = MODE == kModeOutF32 ? 16 : 32;
+    static constexpr int CH = CIN / 8, COUT = MODE == kModeOutF32 || MODE == kModeStart ? 16 : 32;
+    static constexpr int PL = stored_planes(CIN);
     static constexpr int STAGE = (CH * kRowPx * 16 + 127) / 128 * 128;   // one input row with its two halo columns
     static constexpr int WBLK = 2 * 5 * COUT * 16;                       // weights of one (dx, channel half): 5 blocks
     static constexpr int NWB = 3 * (CIN / 16);
@@ -514,9 +533,10 @@ struct RowsCfg {
 template <int CIN, int MODE>
 __global__ void __launch_bounds__(192, 3)
 conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const float* __restrict__ bias,
-             void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, int* __restrict__ err) {
+             void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, int* __restrict__ err,
+             const __grid_constant__ StartOut st) {
     using C = RowsCfg<CIN, MODE>;
-    constexpr int CH = C::CH, COUT = C::COUT, S = kRowStages;
+    constexpr int COUT = C::COUT, PL = C::PL, S = kRowStages;
     extern __shared__ unsigned char rows_raw[];
     __shared__ __align__(8) unsigned long long full[S], empty[S], acc_full[3], acc_empty[3], done;
     __shared__ __align__(16) float smB[32];
@@ -531,7 +551,14 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
         const int dy = (5 - n / COUT) % 3;            // blocks 0..4: 2 1 0 2 1
         cp_async16(smW + (size_t)e * 16, wpk + ((size_t)(dy * 3 + dx) * COUT + co) * CIN + (2 * j + kh) * 8);
     }
-    if (MODE != kModeGateBf16 && tid < (MODE == kModeOutF32 ? kOut : COUT)) smB[tid] = bias[tid];
+    if (MODE != kModeGateBf16 && tid < (COUT == 16 ? kOut : COUT)) smB[tid] = bias[tid];
+    if constexpr (PL < C::CH) {
+        // planes that are not in memory stay zero
+        for (int e = tid; e < S * (C::CH - PL) * kRowPx; e += 192) {
+            const int i = e / ((C::CH - PL) * kRowPx), k = e - i * ((C::CH - PL) * kRowPx);
+            *reinterpret_cast<uint4*>(sm + i * C::STAGE + (PL * kRowPx + k) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sh_addr(&tmem_base)),
                      "n"(C::TMEM_COLS)
@@ -591,15 +618,15 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                     if (!ok) break;
                     used = n - S + 1;
                 }
-                unsigned char* st = sm + s * C::STAGE;
+                unsigned char* sg = sm + s * C::STAGE;
                 const bool inside = r >= 0 && r < H;
                 const int h0 = inside ? lo : kRowPx, nz = kRowPx - (inside ? hi - lo : 0);
                 if (nz > 0) {
                     // zeros outside the image: slots [0, h0) and, for a row inside, [hi, kRowPx)
-                    for (int e = lane; e < nz * CH; e += 32) {
+                    for (int e = lane; e < nz * PL; e += 32) {
                         const int pl = e / nz, k = e - pl * nz;
                         const int slot = k < h0 ? k : hi + (k - h0);
-                        *reinterpret_cast<uint4*>(st + (pl * kRowPx + slot) * 16) = make_uint4(0u, 0u, 0u, 0u);
+                        *reinterpret_cast<uint4*>(sg + (pl * kRowPx + slot) * 16) = make_uint4(0u, 0u, 0u, 0u);
                     }
                     fence_async_shared();
                     __syncwarp();
@@ -608,13 +635,13 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                     const uint32_t bar = sh_addr(&full[s]);
                     if (inside) {
                         const uint32_t bytes = (uint32_t)(hi - lo) * 16u;
-                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes * CH)
+                        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes * PL)
                                      : "memory");
-                        const bf16* src = in + ((size_t)img * CH * hw + (size_t)r * W + c0) * 8;
-                        for (int pl = 0; pl < CH; ++pl)
+                        const bf16* src = in + ((size_t)img * PL * hw + (size_t)r * W + c0) * 8;
+                        for (int pl = 0; pl < PL; ++pl)
                             asm volatile(
                                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                    sh_addr(st + (pl * kRowPx + lo) * 16)),
+                                    sh_addr(sg + (pl * kRowPx + lo) * 16)),
                                 "l"(src + (size_t)pl * hw * 8), "r"(bytes), "r"(bar)
                                 : "memory");
                     } else {
@@ -694,7 +721,7 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                 const int k = (n0 + d + 2) % 3, o = y0 - 2 + d;
                 const bool keep = d >= 2 && d < R + 2 && c < W;
                 // pixel's slot in plane 0 of its image; plane p is p hw slots further
-                const size_t px = (size_t)img * (MODE == kModeOutF32 ? 1 : 4) * hw + (size_t)o * W + c;
+                const size_t px = (size_t)img * (COUT == 16 ? 1 : 4) * hw + (size_t)o * W + c;
                 uint4 gv[4];
                 if constexpr (MODE == kModeGateBf16) {
                     const uint4* gp = reinterpret_cast<const uint4*>(gate) + px;
@@ -713,6 +740,13 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                 if constexpr (MODE == kModeOutF32) {
                     reinterpret_cast<float4*>(out)[px] =
                         make_float4(v[0] + smB[0], v[1] + smB[1], v[2] + smB[2], v[3] + smB[3]);
+                } else if constexpr (MODE == kModeStart) {
+                    const size_t ip = (size_t)o * W + c;
+                    float* x0 = st.separate ? st.px0[img] : st.x0 + (size_t)img * hw;
+                    float* d0 = st.separate ? st.pd0[img] : st.d0 + (size_t)img * 3 * hw;
+                    x0[ip] = st.s0 * (v[0] + smB[0]);
+                    d0[ip] = st.s1 * (v[1] + smB[1]);
+                    reinterpret_cast<float2*>(d0 + hw)[ip] = make_float2(st.s2 * (v[2] + smB[2]), st.s2 * (v[3] + smB[3]));
                 } else {
                     uint4* op = reinterpret_cast<uint4*>(out) + px;
 #pragma unroll
@@ -1064,34 +1098,55 @@ wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ grads, int
 }
 
 // ---------------------------------------------------------------------------
-// loss and its gradient in the output: g = 2 c_k (o - t) / npx (16 channels
-// in two planes, 4 used; hw = H W); per-block FP64 partial sums of the loss
+// loss and its gradient in the output: g = 2 c_k (o - t) / npx (one plane of
+// eight channels, 4 used; its readers take the second plane of a 16-channel
+// operand as zeros outside the tensor map). Bound by its 48 B per pixel. The
+// squared errors are summed per thread as FP32 pairs without rounding error
+// (product and sum split exactly, which keeps about 48 bits: FP64 units are
+// scarce here), per block in FP64, one atomic per block; the grid is a few
+// blocks per SM, not one block per 256 pixels: 4096 atomics on one address and
+// eight FP64 operations per pixel made it 50 us at 16 x 256^2.
 // ---------------------------------------------------------------------------
-__global__ void cnn_loss_kernel(const float* __restrict__ o, const float* __restrict__ tg, float4 cw,
-                                bf16* __restrict__ gout, double* __restrict__ loss, long long npx, long long hw) {
-    __shared__ double red[8];
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (i < npx) {
-        const float4 ov = reinterpret_cast<const float4*>(o)[i];
-        const float4 tv = reinterpret_cast<const float4*>(tg)[i];
-        const float e0 = ov.x - tv.x, e1 = ov.y - tv.y, e2 = ov.z - tv.z, e3 = ov.w - tv.w;
-        l = (double)cw.x * e0 * e0 + (double)cw.y * e1 * e1 + (double)cw.z * e2 * e2 + (double)cw.w * e3 * e3;
-        const float s = 2.0f / (float)npx;
-        const long long img = i / hw, px = i - img * hw;
-        uint4* dst = reinterpret_cast<uint4*>(gout + (img * 2 * hw + px) * 8);
-        dst[0] = make_uint4(pack2(__float2bfloat16(s * cw.x * e0), __float2bfloat16(s * cw.y * e1)),
-                            pack2(__float2bfloat16(s * cw.z * e2), __float2bfloat16(s * cw.w * e3)), 0u, 0u);
-        dst[hw] = make_uint4(0u, 0u, 0u, 0u);
+struct PairSum {
+    float h = 0.f, l = 0.f;
+    // add v * v
+    __device__ __forceinline__ void add_sq(float v) {
+        const float p = v * v, e = fmaf(v, v, -p);
+        const float t = h + p, z = t - h;
+        l += ((h - (t - z)) + (p - z)) + e;
+        h = t;
     }
+    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+};
+
+__global__ void __launch_bounds__(256)
+cnn_loss_kernel(const float* __restrict__ o, const float* __restrict__ tg, float4 cw, bf16* __restrict__ gout,
+                double* __restrict__ loss, long long npx) {
+    __shared__ double red[8];
+    PairSum sx, sy, sz, sw;
+    const float s = 2.0f / (float)npx;
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < npx; i += (long long)gridDim.x * 256) {
+        const float4 ov = reinterpret_cast<const float4*>(o)[i];
+        const float4 tv = __ldcs(reinterpret_cast<const float4*>(tg) + i);
+        const float e0 = ov.x - tv.x, e1 = ov.y - tv.y, e2 = ov.z - tv.z, e3 = ov.w - tv.w;
+        sx.add_sq(e0);
+        sy.add_sq(e1);
+        sz.add_sq(e2);
+        sw.add_sq(e3);
+        reinterpret_cast<uint4*>(gout)[i] =
+            make_uint4(pack2(__float2bfloat16(s * cw.x * e0), __float2bfloat16(s * cw.y * e1)),
+                       pack2(__float2bfloat16(s * cw.z * e2), __float2bfloat16(s * cw.w * e3)), 0u, 0u);
+    }
+    double l = (double)cw.x * sx.value() + (double)cw.y * sy.value() + (double)cw.z * sz.value() +
+               (double)cw.w * sw.value();
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
     __syncthreads();
     if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(loss, s / (double)npx);
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        atomicAdd(loss, t / (double)npx);
     }
 }
 
@@ -1150,7 +1205,6 @@ __global__ void split_start_kernel(const float* __restrict__ o, float s0, float 
 
 // the same two steps for a group of separately stored problems (the learned
 // start of a batch solve): per-image device pointers, passed by value
-constexpr int kWsBatch = 16;
 struct ImgPtrs {
     const float* y[kWsBatch];
     const uint8_t* m[kWsBatch];
@@ -1250,8 +1304,9 @@ cudaError_t conv_tc(bool first, const bf16* in, const bf16* w, const float* bias
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap tm;
     const cuuint64_t plane = (cuuint64_t)W * H * 16;
-    const cuuint64_t dims[4] = {(cuuint64_t)W * 8, (cuuint64_t)H, (cuuint64_t)(CIN / 8), (cuuint64_t)count};
-    const cuuint64_t strides[3] = {(cuuint64_t)W * 16, plane, plane * (CIN / 8)};
+    constexpr int PL = stored_planes(CIN);       // (a plane outside the map reads as zero)
+    const cuuint64_t dims[4] = {(cuuint64_t)W * 8, (cuuint64_t)H, (cuuint64_t)PL, (cuuint64_t)count};
+    const cuuint64_t strides[3] = {(cuuint64_t)W * 16, plane, plane * PL};
     const cuuint32_t box[4] = {(cuuint32_t)kTcHW * 8, (cuuint32_t)kTcHH, (cuuint32_t)(CIN / 8), 1};
     const cuuint32_t es[4] = {1, 1, 1, 1};
     if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(in), dims, strides, box, es,
@@ -1273,10 +1328,12 @@ bool rows_fit(int W) { return ((W + kStrip - 1) / kStrip) * kStrip * 4 <= W * 5;
 // columns fit the width, else the 8 x 16 tiles of conv3x3_tc
 template <int CIN, int MODE>
 cudaError_t conv_rows(const bf16* in, const bf16* w, const float* bias, void* out, const bf16* gate, int count,
-                      int H, int W, int sms, int* err, cudaStream_t s) {
+                      int H, int W, int sms, int* err, cudaStream_t s, const StartOut& st = StartOut{}) {
     using C = RowsCfg<CIN, MODE>;
     const int strips = (W + kStrip - 1) / kStrip;
-    if (!rows_fit(W)) return conv_tc<CIN, MODE>(false, in, w, bias, out, gate, count, H, W, sms, err, s);
+    if constexpr (MODE != kModeStart) {
+        if (!rows_fit(W)) return conv_tc<CIN, MODE>(false, in, w, bias, out, gate, count, H, W, sms, err, s);
+    }
     cudaError_t e = cudaFuncSetAttribute(conv3x3_rows<CIN, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)C::SMEM);
     if (e == cudaSuccess)
@@ -1286,7 +1343,8 @@ cudaError_t conv_rows(const bf16* in, const bf16* w, const float* bias, void* ou
     // (at least eight strip rows per CTA: each segment adds two halo rows)
     const long long total = (long long)count * strips * H;
     const int grid = (int)std::max(1LL, std::min((long long)C::CTAS * sms, total / 8));
-    return launch_layer(conv3x3_rows<CIN, MODE>, false, grid, 192, C::SMEM, s, in, w, bias, out, gate, H, W, count, err);
+    return launch_layer(conv3x3_rows<CIN, MODE>, false, grid, 192, C::SMEM, s, in, w, bias, out, gate, H, W, count, err,
+                        st);
 }
 
 // One layer's weight and bias gradients into the CTAs' partial vectors. The
@@ -1336,7 +1394,7 @@ struct admm_cnn_s {
     bf16* act[kLayers - 1] = {};   // activations after layers 0..6 (training keeps all)
     float* out = nullptr;          // output, 4 channels FP32
     bf16* gbuf[2] = {};            // gradient ping-pong, 32 channels
-    bf16* gout = nullptr;          // output gradient, 16 channels
+    bf16* gout = nullptr;          // output gradient, one plane of 8 channels
     float* wpart = nullptr;        // weight-gradient partial vectors, one per CTA and layer
     double* loss = nullptr;        // device accumulator
     double* h_loss = nullptr;      // pinned
@@ -1380,13 +1438,19 @@ int pack_all(admm_cnn_s* n, cudaStream_t s) {
 }
 
 // the eight layers on the prepared input n->a0; with `keep` every activation
-// is stored for the backward pass, otherwise two buffers alternate
-int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, cudaStream_t s) {
+// is stored for the backward pass, otherwise two buffers alternate. The output
+// goes to `out` (16-byte aligned) or, with `st` (rows_fit(W) only), to a
+// predicted start.
+int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, float* out, const StartOut* st, cudaStream_t s) {
     const bf16* cur = n->a0;
     for (int l = 0; l < kLayers; ++l) {
         const float* b = n->params + param_offset(l) + (long long)layer_cout(l) * layer_cin(l) * 9;
         if (l == kLayers - 1) {
-            CKC((conv_rows<32, kModeOutF32>(cur, n->wf[l], b, n->out, nullptr, count, H, W, n->sms, n->tc_err, s)));
+            if (st)
+                CKC((conv_rows<32, kModeStart>(cur, n->wf[l], b, nullptr, nullptr, count, H, W, n->sms, n->tc_err, s,
+                                               *st)));
+            else
+                CKC((conv_rows<32, kModeOutF32>(cur, n->wf[l], b, out, nullptr, count, H, W, n->sms, n->tc_err, s)));
         } else {
             bf16* dst = keep ? n->act[l] : n->act[l & 1];
             if (l == 0)
@@ -1400,13 +1464,13 @@ int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, cudaStream_t s
 }
 
 // forward pass from [M^T y, mask] stored contiguously for the count images
-int forward(admm_cnn_s* n, int count, int H, int W, const float* ybar, const uint8_t* mask, bool keep,
-            cudaStream_t s) {
+int forward(admm_cnn_s* n, int count, int H, int W, const float* ybar, const uint8_t* mask, bool keep, float* out,
+            const StartOut* st, cudaStream_t s) {
     const long long npx = (long long)count * H * W;
     cnn_input_kernel<<<(unsigned)((npx + 255) / 256), 256, 0, s>>>(ybar, mask, n->a0, npx);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
-    return run_layers(n, count, H, W, keep, s);
+    return run_layers(n, count, H, W, keep, out, st, s);
 }
 
 // loss, gradients into n->grads
@@ -1414,8 +1478,8 @@ int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const 
     const long long npx = (long long)count * H * W;
     CKC(cudaMemsetAsync(n->loss, 0, sizeof(double), s));
     const float4 cw = make_float4(chan_w[0], chan_w[1], chan_w[2], chan_w[3]);
-    cnn_loss_kernel<<<(unsigned)((npx + 255) / 256), 256, 0, s>>>(n->out, target, cw, n->gout, n->loss, npx,
-                                                                   (long long)H * W);
+    const unsigned lgrid = (unsigned)std::min((npx + 255) / 256, 6LL * n->sms);
+    cnn_loss_kernel<<<lgrid, 256, 0, s>>>(n->out, target, cw, n->gout, n->loss, npx);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
     const int tiles = ((H + kWgTH - 1) / kWgTH) * ((W + kWgTW - 1) / kWgTW) * count;
@@ -1439,7 +1503,7 @@ int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const 
         float* pt = n->wpart + ra.base[l] * ncta;
         const bf16* a_in = l == 0 ? n->a0 : n->act[l - 1];
         if (l == kLayers - 1)
-            CKC((wgrad<false, 4, 2>(true, a_in, g, pt, kWidth, kOut, count, H, W, ncta, n->tc_err, s)));
+            CKC((wgrad<false, 4, 1>(true, a_in, g, pt, kWidth, kOut, count, H, W, ncta, n->tc_err, s)));
         else if (l == 0)
             CKC((wgrad<true, 1, 4>(false, a_in, g, pt, kIn, kWidth, count, H, W, ncta, n->tc_err, s)));
         else
@@ -1506,7 +1570,7 @@ int admm_cnn_create(admm_cnn_t* out, long long max_pixels, int training) {
     if (n->training) {
         if ((rc = dalloc(n, &n->grads, P)) || (rc = dalloc(n, &n->m, P)) || (rc = dalloc(n, &n->v, P)) ||
             (rc = dalloc(n, &n->gbuf[0], px * kWidth)) || (rc = dalloc(n, &n->gbuf[1], px * kWidth)) ||
-            (rc = dalloc(n, &n->gout, px * 16)) || (rc = dalloc(n, &n->loss, 1)) ||
+            (rc = dalloc(n, &n->gout, px * 8)) || (rc = dalloc(n, &n->loss, 1)) ||
             (rc = dalloc(n, &n->wpart, (size_t)P * n->sms)))
             return bail(rc);
         if (admm::alloc_fault_fire() || cudaHostAlloc(&n->h_loss, sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
@@ -1551,8 +1615,11 @@ int admm_cnn_forward(admm_cnn_t net, int count, int H, int W, const float* ybar,
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if ((rc = forward(net, count, H, W, ybar, mask, false, s)) != ADMM_OK) return rc;
-    CKC(cudaMemcpyAsync(out, net->out, (size_t)count * H * W * 4 * sizeof(float), cudaMemcpyDeviceToDevice, s));
+    // (the last layer stores 16 bytes per pixel: straight to `out` where that is aligned)
+    const bool direct = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+    if ((rc = forward(net, count, H, W, ybar, mask, false, direct ? out : net->out, nullptr, s)) != ADMM_OK) return rc;
+    if (!direct)
+        CKC(cudaMemcpyAsync(out, net->out, (size_t)count * H * W * 4 * sizeof(float), cudaMemcpyDeviceToDevice, s));
     return ADMM_OK;
 }
 
@@ -1563,7 +1630,7 @@ int admm_cnn_gradients(admm_cnn_t net, int count, int H, int W, const float* yba
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if ((rc = forward(net, count, H, W, ybar, mask, true, s)) != ADMM_OK) return rc;
+    if ((rc = forward(net, count, H, W, ybar, mask, true, net->out, nullptr, s)) != ADMM_OK) return rc;
     if ((rc = backward(net, count, H, W, target, chan_w, s)) != ADMM_OK) return rc;
     CKC(cudaMemcpyAsync(grads, net->grads, param_count() * sizeof(float), cudaMemcpyDefault, s));
     CKC(cudaMemcpyAsync(net->h_loss, net->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -1579,7 +1646,7 @@ int admm_cnn_train_step(admm_cnn_t net, int count, int H, int W, const float* yb
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if ((rc = forward(net, count, H, W, ybar, mask, true, s)) != ADMM_OK) return rc;
+    if ((rc = forward(net, count, H, W, ybar, mask, true, net->out, nullptr, s)) != ADMM_OK) return rc;
     if ((rc = backward(net, count, H, W, target, chan_w, s)) != ADMM_OK) return rc;
     net->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
@@ -1606,7 +1673,15 @@ int admm_cnn_predict_start(admm_cnn_t net, int count, int H, int W, const float*
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    if ((rc = forward(net, count, H, W, ybar, mask, false, s)) != ADMM_OK) return rc;
+    StartOut st{};
+    st.s0 = scales[0];
+    st.s1 = scales[1];
+    st.s2 = scales[2];
+    st.x0 = x0;
+    st.d0 = d0;
+    const bool fit = rows_fit(W);
+    if ((rc = forward(net, count, H, W, ybar, mask, false, net->out, fit ? &st : nullptr, s)) != ADMM_OK) return rc;
+    if (fit) return ADMM_OK;         // the last layer has written the start
     const long long n = (long long)H * W, npx = n * count;
     split_start_kernel<<<(unsigned)((npx + 255) / 256), 256, 0, s>>>(net->out, scales[0], scales[1], scales[2], x0,
                                                                      d0, n, npx);
@@ -1736,7 +1811,18 @@ int ws_predict_starts(int count, int H, int W, const float* const* ybar, const u
     cnn_input_ptrs_kernel<<<grid, 256, 0, s>>>(P, net->a0, hw);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
-    if ((rc = run_layers(net, count, H, W, false, s)) != ADMM_OK) return rc;
+    StartOut st{};
+    st.s0 = g_ws.scales[0];
+    st.s1 = g_ws.scales[1];
+    st.s2 = g_ws.scales[2];
+    st.separate = 1;
+    for (int i = 0; i < count; ++i) {
+        st.px0[i] = x0[i];
+        st.pd0[i] = d0[i];
+    }
+    const bool fit = rows_fit(W);
+    if ((rc = run_layers(net, count, H, W, false, net->out, fit ? &st : nullptr, s)) != ADMM_OK) return rc;
+    if (fit) return ADMM_OK;         // the last layer has written the starts
     split_start_ptrs_kernel<<<grid, 256, 0, s>>>(net->out, g_ws.scales[0], g_ws.scales[1], g_ws.scales[2], P, hw);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
