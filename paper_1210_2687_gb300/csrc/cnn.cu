@@ -33,6 +33,7 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/admm_warmstart.h"
@@ -80,6 +81,40 @@ int fail(cudaError_t) { return ADMM_ECUDA; }
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+}
+
+// a + b of both FP32 halves
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t pair2(float lo, float hi) {
+    return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);
+}
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
+// (lo, hi) rounded to BF16
+__device__ __forceinline__ uint32_t cvt2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+// max(., 0) of both BF16 halves (NaN gives 0, as fmaxf does)
+__device__ __forceinline__ uint32_t relu2(uint32_t v) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0u));
+    return r;
+}
+// all ones in each half whose BF16 value is > 0
+__device__ __forceinline__ uint32_t positive2(uint32_t v) {
+    uint32_t r;
+    asm("set.gt.u32.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0u));
+    return r;
 }
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -181,22 +216,29 @@ __device__ __forceinline__ unsigned long long gtimer_ns() {
     return t;
 }
 
-// wait for phase `parity` of the mbarrier, at most about a second; try_wait
-// suspends the thread in hardware until the phase completes or a short
-// hardware time limit passes, so the loop does not spin
+// Wait for phase `parity` of the mbarrier, at most about a second. try_wait
+// suspends the thread in hardware until the phase completes or the time limit
+// given here (1 ms) passes, so the loop does not poll: a poll is a
+// shared-memory access, and the tensor cores need that bandwidth. The clock is
+// read only after a failed try: %globaltimer takes hundreds of cycles, and most
+// waits find their phase complete.
+__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(mbar), "r"(parity), "r"(1000000u)
+        : "memory");
+    return done != 0;
+}
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity) {
+    if (mbar_try(mbar, parity)) return true;
     const unsigned long long t0 = gtimer_ns();
-    for (;;) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (gtimer_ns() - t0 > 1000000000ull) return false;
-    }
+    do {
+        if (mbar_try(mbar, parity)) return true;
+    } while (gtimer_ns() - t0 <= 1000000000ull);
+    return false;
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -654,50 +696,67 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
         // every stage's last release has arrived before the CTA ends
         for (int k = max(0, n - S); ok && k < n; ++k)
             ok = mbar_wait_bounded(sh_addr(&empty[k % S]), (uint32_t)((k / S) & 1));
-    } else if (warp == 1 && lane == 0) {
-        int n = 0;
-        uint32_t eph = 0, need = 7;                  // slots whose clearing is not yet seen (at first: all)
-        const uint32_t wB = sh_addr(smW);
-        auto slot_clear = [&](int k) -> bool {
+    } else if (warp == 1) {
+        // The warp stays converged and one lane is elected around the issue
+        // itself, so that the descriptors are uniform values; their start
+        // address is the lowest field, in units of 16 bytes.
+        const uint64_t a_in = umma_desc(sh_addr(sm), kRowPx * 16, 128);
+        const uint64_t b_in = umma_desc(sh_addr(smW), 5 * COUT * 16, 128);
+        uint32_t s = 0, fp = 0, eph = 0, need = 7;   // stage and phase; slots whose clearing is not yet seen (at first: all)
+        auto slot_clear = [&](uint32_t k) -> bool {
             if (!((need >> k) & 1u)) return true;
             if (!mbar_wait_bounded(sh_addr(&acc_empty[k]), (eph >> k) & 1u)) return false;
             eph ^= 1u << k;
             need &= ~(1u << k);
             return true;
         };
+        // one input row in the rotation PH of the slots
+        auto row = [&](auto rotation, bool first, bool last) -> bool {
+            constexpr int PH = decltype(rotation)::value, UP = (PH + 1) % 3, DOWN = (PH + 2) % 3;   // slots of rows r + 1, r - 1
+            if (!mbar_wait_bounded(sh_addr(&full[s]), fp) || !slot_clear(UP) ||
+                (first && !(slot_clear(PH) && slot_clear(DOWN))))
+                return false;
+            tc_fence_after();
+            const uint64_t a0 = a_in + s * (C::STAGE / 16);
+            const uint64_t b0 = b_in + (PH == 0 ? 1 : (PH == 1 ? 0 : 2)) * COUT;         // window start
+            if (elect_one()) {
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                    for (int j = 0; j < CIN / 16; ++j)
+                        umma_f16(tmem, a0 + (2 * j * kRowPx + dx), b0 + (dx * (CIN / 16) + j) * (C::WBLK / 16),
+                                 idesc_m128(C::N), 1u);
+                }
+                commit(&acc_full[DOWN]);             // output row r - 1 is complete
+                commit(&empty[s]);
+                if (last) {
+                    // the two rows that the segment's last input row has begun are dropped
+                    commit(&acc_full[PH]);
+                    commit(&acc_full[UP]);
+                }
+            }
+            __syncwarp();
+            need |= last ? 7u : 1u << DOWN;
+            if (++s == S) {
+                s = 0;
+                fp ^= 1u;
+            }
+            return true;
+        };
         for (long long pos = a0; pos < a1 && ok;) {
             const int y0 = (int)(pos % H);
             const int R = (int)min((long long)(H - y0), a1 - pos);
             pos += R;
-            for (int i = 0; i < R + 2; ++i, ++n) {
-                const int s = n % S, ph = n % 3;
-                // (first row of a segment: all three slots)
-                ok = mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((n / S) & 1)) && slot_clear((ph + 1) % 3) &&
-                     (i > 0 || (slot_clear(ph) && slot_clear((ph + 2) % 3)));
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t aB = sh_addr(sm + s * C::STAGE);
-                const uint32_t w0 = wB + (uint32_t)((4 - ph) % 3) * (COUT * 16);   // window start: 1, 0, 2
-#pragma unroll
-                for (int dx = 0; dx < 3; ++dx) {
-#pragma unroll
-                    for (int j = 0; j < CIN / 16; ++j) {
-                        const uint64_t a = umma_desc(aB + (2 * j * kRowPx + dx) * 16, kRowPx * 16, 128);
-                        const uint64_t b = umma_desc(w0 + (dx * (CIN / 16) + j) * C::WBLK, 5 * COUT * 16, 128);
-                        umma_f16(tmem, a, b, idesc_m128(C::N), 1u);
-                    }
-                }
-                commit(&empty[s]);
-                commit(&acc_full[(ph + 2) % 3]);     // output row r - 1 is complete
-                need |= 1u << ((ph + 2) % 3);
+            // (every segment starts in rotation 0)
+            const int n = R + 2;
+            for (int t = 0; t < n && ok; t += 3) {
+                ok = row(std::integral_constant<int, 0>(), t == 0, t + 1 == n);
+                if (ok && t + 1 < n) ok = row(std::integral_constant<int, 1>(), false, t + 2 == n);
+                if (ok && t + 2 < n) ok = row(std::integral_constant<int, 2>(), false, t + 3 == n);
             }
-            if (!ok) break;
-            // the two rows that the segment's last input row has begun are dropped
-            commit(&acc_full[(n - 1) % 3]);
-            commit(&acc_full[n % 3]);
-            need = 7;
         }
-        commit(&done);
+        ok = __all_sync(0xffffffffu, ok);
+        if (elect_one()) commit(&done);              // (the thread that has issued the MMAs)
     } else if (warp >= 2) {
         const int q = warp & 3;                      // this warp's quarter of the tensor-memory lanes
         const uint32_t tw = tmem + ((uint32_t)(32 * q) << 16);
@@ -709,7 +768,11 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
             if (lane == 0) arrive(&acc_empty[k]);
         };
         for (int k = 0; k < 3; ++k) release(k);
-        int n0 = 0;
+        uint64_t bs[COUT / 2];                       // bias pairs
+        if constexpr (MODE == kModeReluBf16) {
+#pragma unroll
+            for (int h = 0; h < COUT / 2; ++h) bs[h] = pair2(smB[2 * h], smB[2 * h + 1]);
+        }
         uint32_t fph = 0;
         for (long long pos = a0; pos < a1 && ok;) {
             const int col = (int)(pos / H), y0 = (int)(pos - (long long)col * H);
@@ -717,8 +780,9 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
             const int img = col / strips, xs = (col - img * strips) * kStrip;
             pos += R;
             const int c = xs + 32 * q + lane;
-            for (int d = 0; d < R + 4; ++d) {
-                const int k = (n0 + d + 2) % 3, o = y0 - 2 + d;
+            int k = 2;                               // slot of the drain: (d + 2) mod 3
+            for (int d = 0; d < R + 4; ++d, k = k == 2 ? 0 : k + 1) {
+                const int o = y0 - 2 + d;
                 const bool keep = d >= 2 && d < R + 2 && c < W;
                 // pixel's slot in plane 0 of its image; plane p is p hw slots further
                 const size_t px = (size_t)img * (COUT == 16 ? 1 : 4) * hw + (size_t)o * W + c;
@@ -753,27 +817,21 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                     for (int p = 0; p < 4; ++p) {
                         uint32_t pk[4];
                         if constexpr (MODE == kModeReluBf16) {
-                            const float4 b0 = *reinterpret_cast<const float4*>(smB + 8 * p);
-                            const float4 b1 = *reinterpret_cast<const float4*>(smB + 8 * p + 4);
-                            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-                            for (int h = 0; h < 4; ++h)
-                                pk[h] = pack2(__float2bfloat16(fmaxf(v[8 * p + 2 * h] + b[2 * h], 0.f)),
-                                              __float2bfloat16(fmaxf(v[8 * p + 2 * h + 1] + b[2 * h + 1], 0.f)));
+                            for (int h = 0; h < 4; ++h) {
+                                const uint64_t u = add2(pair2(v[8 * p + 2 * h], v[8 * p + 2 * h + 1]), bs[4 * p + h]);
+                                pk[h] = relu2(cvt2(__uint_as_float((uint32_t)u), __uint_as_float((uint32_t)(u >> 32))));
+                            }
                         } else {
                             const uint32_t gw[4] = {gv[p].x, gv[p].y, gv[p].z, gv[p].w};
 #pragma unroll
-                            for (int h = 0; h < 4; ++h) {
-                                const float g0 = __uint_as_float(gw[h] << 16), g1 = __uint_as_float(gw[h] & 0xFFFF0000u);
-                                pk[h] = pack2(__float2bfloat16(g0 > 0.f ? v[8 * p + 2 * h] : 0.f),
-                                              __float2bfloat16(g1 > 0.f ? v[8 * p + 2 * h + 1] : 0.f));
-                            }
+                            for (int h = 0; h < 4; ++h)
+                                pk[h] = cvt2(v[8 * p + 2 * h], v[8 * p + 2 * h + 1]) & positive2(gw[h]);
                         }
                         op[p * hw] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                     }
                 }
             }
-            n0 += R + 2;
         }
     }
     __syncwarp();
