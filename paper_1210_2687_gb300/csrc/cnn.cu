@@ -679,12 +679,17 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                         const uint32_t bytes = (uint32_t)(hi - lo) * 16u;
                         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes * PL)
                                      : "memory");
+                        // read once here: what stays in L2 is the output, which the next layer reads
+                        // (at 16 x 256^2, where it fits, 834 -> 807 us for loss and gradients)
+                        uint64_t once;
+                        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
                         const bf16* src = in + ((size_t)img * PL * hw + (size_t)r * W + c0) * 8;
                         for (int pl = 0; pl < PL; ++pl)
                             asm volatile(
-                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, "
+                                "[%3], %4;" ::"r"(
                                     sh_addr(sg + (pl * kRowPx + lo) * 16)),
-                                "l"(src + (size_t)pl * hw * 8), "r"(bytes), "r"(bar)
+                                "l"(src + (size_t)pl * hw * 8), "r"(bytes), "r"(bar), "l"(once)
                                 : "memory");
                     } else {
                         arrive(&full[s]);

@@ -30,6 +30,7 @@
 #include "haar.cuh"
 #include "cg.cuh"
 #include "gen.cuh"
+#include "team.cuh"
 #include "setup.cuh"
 #include "variants.cuh"
 
@@ -146,6 +147,7 @@ struct Profile {
 long long g_launches = 0;            // every kernel launched (under g_mutex)
 int g_max_slots = 0;                 // ADMM_OPT_MAX_SLOTS
 int g_test_stall = 0;                // ADMM_OPT_TEST_STALL: armed for the next solve
+thread_local bool t_general = false; // the autotuner's trials: the general kernels it compares
 
 int prof_event(size_t i, cudaStream_t s) {
     while (g_prof.ev.size() <= i) {
@@ -652,7 +654,7 @@ int admm_deconv_plan(admm_plan_t* out, const admm_params_t* p, void* stream) {
     const size_t omk = take(n);
     const size_t olm = take((size_t)pl->Wc * H * sizeof(float2));
     const size_t okt = take((size_t)pl->Wc * H * sizeof(float));
-    const size_t opt = take((size_t)pl->n_slots * kNumPartials * sizeof(double));
+    const size_t opt = take((size_t)std::max(pl->n_slots, kMaxTeam) * kNumPartials * sizeof(double));
     const size_t oct = take(sizeof(ProbCtl));
     const size_t oys = take(n * sizeof(float));
     const size_t oms = take(n);
@@ -950,6 +952,19 @@ int admm_deconv_set_state(admm_plan_t plan, const float* state, void* stream) {
     return ADMM_OK;
 }
 
+// Whether `count` problems of a small TV class run on teams: as many as are
+// resident at once, or twice that with clusters (a second round of teams, which
+// the hardware starts as the first ones end). Beyond it the general kernels,
+// whose iteration costs about the same for one image as for a few dozen, are
+// faster. Per iteration of the whole batch, team / general: 64 x 64: 1 image 3.9
+// / 19.2 us, 32: 5.9 / 25, 64 (two rounds): 12 / 25; 128 x 128: 1: 5.7 / 20, 16
+// (two rounds): 14 / 24, 32 (four): 28 / 28; 256 x 256: 1: 8.5 / 18.4, 4 (two
+// rounds): 17 / 18.7.
+static bool use_tv_team(int H, int W, bool aniso, int count) {
+    const int cap = tv_team_capacity(H, W, aniso);
+    return count <= cap * (tv_team_cluster(H, W) ? 2 : 1);
+}
+
 // One size class of a batch: problems [off, off + count) of the descriptor
 // table, split into L.n lanes (absolute table offsets and slot ranges; lane l
 // uses queue word qbase + l).
@@ -1098,6 +1113,13 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
     std::vector<int> order;                       // table position -> index into plans
     std::vector<char> x_host;
     int soff = 0, qbase = 0;
+    // A call of one class of small TV images runs each image on a team of CTAs,
+    // many iterations per launch (team.cuh): not with per-phase timing, whose
+    // phases are the general kernels', nor with the stall hook, which withholds
+    // one of their copies; and only in the row configuration whose bits the team
+    // kernel reproduces, so that a problem's result does not depend on how many
+    // are solved with it.
+    bool team = classes.size() == 1 && !prof && !t_general && g_test_stall == 0;
     // input preparation, batched: items [prep_done, prep_n) of the pinned
     // staging table are prepared by the next flush (before a learned start
     // reads its problem's prepared input, and after the last problem)
@@ -1235,7 +1257,10 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
         g.nslots = choose_slots(g.H, g.W, g.tv, g.R, g.slot_ctas, g.count);
         // with per-phase timing on, one lane: every launch covers all slots,
         // so the timed phases are the full-size kernels
-        g.L.n = prof ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : kDefaultLanes, g.count, g.nslots}));
+        // (as is a class that runs in teams)
+        team = team && g.tv && !g.gen && g.row_v == 0 && g.nslots == g.count &&
+               use_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, g.count);
+        g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : kDefaultLanes, g.count, g.nslots}));
         for (int l = 0, o = g.off, so = soff; l < g.L.n; ++l) {
             g.L.off[l] = o;
             g.L.cnt[l] = l + 1 < g.L.n ? g.count / g.L.n : g.off + g.count - o;
@@ -1290,6 +1315,16 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
     if (prof) {
         int r = prof_event(nev++, s);
         if (r != ADMM_OK) return r;
+    }
+    while (team && !live.empty()) {
+        GroupRun& g = live[0];
+        CK(launch_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, ctx->desc + g.off, lane_slots(ctx, g, 0), g.nslots, g.Wp,
+                          ctx->tw, ctx->n_active + g.gi, kTeamSteps, s));
+        ++g_launches;
+        g.launched += kTeamSteps;
+        CK(cudaMemcpyAsync(ctx->h_active, ctx->n_active, sizeof(int), cudaMemcpyDeviceToHost, s));
+        CK(cudaStreamSynchronize(s));
+        if (ctx->h_active[0] <= 0 || g.launched >= g.launch_cap) live.clear();
     }
     for (int j = 0; !live.empty(); ++j) {
         bool full = true;
@@ -1634,7 +1669,12 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
         std::vector<float*> xs(problems);
         for (int i = 0; i < problems; ++i) xs[i] = dx + (size_t)i * n;
         // one timed trial of configuration t (installed for the class while it runs)
+        struct General {
+            General() { t_general = true; }
+            ~General() { t_general = false; }
+        };
         auto trial = [&](admm_tuning_t t) -> int {
+            General general;
             describe_tuning(&t);
             {
                 std::lock_guard<std::mutex> lk(g_mutex);

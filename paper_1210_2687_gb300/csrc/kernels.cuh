@@ -50,6 +50,8 @@ struct ProbCtl {
     int pad_;
     unsigned cg_arrive;  // Reeves-Sorel variants: row CTAs that have added their share of alpha's denominator
     float cg_alpha;      // ... and the step of the iteration's conjugate-gradient update
+    unsigned team_bar;           // arrivals at the barriers of tv_team (team.cuh),
+    unsigned team_base;          // and their number when the launch began
     unsigned long long t0;       // device clock (ns) when the batch was set up
     unsigned long long t_start;  // ... when the problem took a slot
     unsigned long long t_done;   // ... when it retired
