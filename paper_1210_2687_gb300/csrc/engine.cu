@@ -121,7 +121,7 @@ struct DeviceCtx {
     // chunk graphs keyed by the batch's layout (size classes, offsets, slots,
     // lanes); cleared whenever the descriptor or slot tables move
     std::map<std::string, cudaGraphExec_t> graphs;
-    // mixed-radix twiddles exp(-2 pi i k / N), k < N, per length N
+    // mixed-radix twiddles per length (fill_gen_table)
     std::map<int, float2*> gtw;
 };
 
@@ -293,12 +293,12 @@ int gen_twiddles(DeviceCtx* c, int N, const float2** out) {
         *out = it->second;
         return ADMM_OK;
     }
-    std::vector<float2> tw(N);
-    for (int k = 0; k < N; ++k) {
-        // exact reduction: angle = 2 pi k / N
-        const double a = 2.0 * M_PI * (double)k / (double)N;
-        tw[k] = make_float2((float)std::cos(a), (float)(-std::sin(a)));
+    if (gfft_odd(N) == 1) {
+        *out = c->tw;                // (radix-8 transforms from the common table)
+        return ADMM_OK;
     }
+    std::vector<float2> tw(N, make_float2(0.f, 0.f));
+    fill_gen_table(N, tw.data());
     float2* t = nullptr;
     CK(dev_alloc(&t, (size_t)N * sizeof(float2)));
     if (cudaMemcpy(t, tw.data(), (size_t)N * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess) {

@@ -71,7 +71,7 @@ gcol_phase(const ProbDesc* __restrict__ probs, SlotTable sl, int Wc, int Wp, con
         const int r = e / CB, c = e % CB;
         cp_async16(stage + e, P.Sb + (size_t)r * Wp + c0 + c);
     }
-    for (int e = tid; e < H / 2; e += kThreads) cp_async16(tw + 2 * e, twH + 2 * e);
+    load_gen_twiddles<H>(tw, twH, tid, kThreads);
 #pragma unroll 1
     for (int c = 0; c < CB; ++c) {
         if (c0 + c >= Wc) break;
@@ -85,7 +85,8 @@ gcol_phase(const ProbDesc* __restrict__ probs, SlotTable sl, int Wc, int Wp, con
     __syncthreads();
     const int kc = c0 + g;
     const bool spec = kc < Wc;
-    float2 v[E], u[E];
+    float2 s2[2][E];                             // the two signals of this column
+    float2 (&v)[E] = s2[0], (&u)[E] = s2[1];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const float4 f = stage[(t + T * e) * CB + g];
@@ -94,9 +95,7 @@ gcol_phase(const ProbDesc* __restrict__ probs, SlotTable sl, int Wc, int Wp, con
     }
     __syncthreads();                             // every column is in registers: the tile is free
     float2* bv = reinterpret_cast<float2*>(stage) + (size_t)(2 * g) * H;
-    float2* bu = bv + H;
-    gfft<H, -1>(v, t, g, tw, bv);
-    gfft<H, -1>(u, t, g, tw, bu);
+    gfft_signals<H, -1>(s2, t, g, tw, bv);
     if (spec) {
         const float2* lcol = lks + g * H;
         const float* kcol = kks + g * H;
@@ -110,8 +109,7 @@ gcol_phase(const ProbDesc* __restrict__ probs, SlotTable sl, int Wc, int Wp, con
             u[e] = cmul(L, xh);
         }
     }
-    gfft<H, 1>(v, t, g, tw, bv);
-    gfft<H, 1>(u, t, g, tw, bu);
+    gfft_signals<H, 1>(s2, t, g, tw, bv);
     __syncthreads();                             // every group is done exchanging through the tile
 #pragma unroll
     for (int e = 0; e < E; ++e) stage[(t + T * e) * CB + g] = make_float4(v[e].x, v[e].y, u[e].x, u[e].y);
@@ -160,12 +158,12 @@ grow_inv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, const 
         cp_async4(pyb + c, P.ybar + pix);
         if (chk && !first) cp_async4(pxp + c, P.xprev + pix);
     }
+    load_gen_twiddles<W>(tw, twW, tid, kThreads);
     cp_async_commit();
-    for (int e = tid; e < W; e += kThreads) tw[e] = twW[e];
-    __syncthreads();
     // the full spectrum of the complex row x + i A x from the two stored halves
     const float4* __restrict__ srow = P.Sa + (size_t)q * Wp;
-    float2 v[E];
+    float2 s1[1][E];
+    float2 (&v)[E] = s1[0];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int kk = t + T * e;
@@ -177,8 +175,9 @@ grow_inv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, const 
             v[e] = make_float2(s.x + s.w, s.z - s.y);
         }
     }
-    gfft<W, 1>(v, t, g, tw, buf + (size_t)g * W);
-    cp_async_wait<0>();          // this thread's staged inputs have landed
+    cp_async_wait<0>();          // the twiddles, and this thread's staged inputs
+    __syncthreads();
+    gfft_signals<W, 1>(s1, t, g, tw, buf + (size_t)g * W);
     float* __restrict__ xw = P.work;
     float* __restrict__ z1w = P.work + n;
     const float mu1 = P.mu1, inv1 = P.inv1pmu1;
@@ -259,16 +258,19 @@ grow_fwd(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, const 
     float2* tw = buf + G * W;
     const int tid = threadIdx.x, g = tid / T, t = tid % T;
     const int q = blockIdx.x * G + g;
-    for (int e = tid; e < W; e += kThreads) tw[e] = twW[e];
-    __syncthreads();
-    float2 v[E];
+    load_gen_twiddles<W>(tw, twW, tid, kThreads);
+    float2 s1[1][E];
+    float2 (&v)[E] = s1[0];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const size_t pix = (size_t)q * W + t + T * e;
         v[e] = make_float2(za[pix], WARM ? 0.f : wb[pix]);
     }
+    cp_async_wait<0>();
+    __syncthreads();
     float2* row = buf + (size_t)g * W;
-    gfft<W, -1>(v, t, g, tw, row);
+    gfft_signals<W, -1>(s1, t, g, tw, row);
+    ggroup_sync<T>(g);
 #pragma unroll
     for (int e = 0; e < E; ++e) row[t + T * e] = v[e];
     ggroup_sync<T>(g);
