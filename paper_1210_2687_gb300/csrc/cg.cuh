@@ -75,23 +75,33 @@ cg_row_a(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, const 
     const int tid = threadIdx.x, g = tid / FT, t = tid % FT;
     const int q = blockIdx.x * G + g;
     const size_t n = (size_t)H * W;
-    load_twiddles<W>(tw, tw_g, tid, kThreads);
-    __syncthreads();
-    float2 v[8];
-    load_row_xax<W>(v, P.Sa + (size_t)q * Wp, t);
-    float2* row = buf + g * W;
-    fft_group<W, 1>(v, row, tw, t, g);
     float* __restrict__ X = P.cg;
     float* __restrict__ AX = P.cg + n;
     float* __restrict__ Sv = P.cg + 4 * n;
     const float* __restrict__ Z = P.cg + 5 * n;
+    const float* __restrict__ Y = P.ybar;
+    // everything the CTA reads is requested before the transform: a load between
+    // the stores below would wait for each of them in turn (eight latencies)
+    float2 v[8];
+    float yb[8], z[8];
+    load_row_xax<W>(v, P.Sa + (size_t)q * Wp, t);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const size_t pix = (size_t)q * W + t + m * FT;
+        yb[m] = Y[pix];
+        z[m] = cold ? 0.f : Z[pix];
+    }
+    load_twiddles<W>(tw, tw_g, tid, kThreads);
+    __syncthreads();
+    float2* row = buf + g * W;
+    fft_group<W, 1>(v, row, tw, t, g);
     CompSum ss;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
         const size_t pix = (size_t)q * W + t + m * FT;
         const float x = v[m].x, ax = v[m].y;
-        const bool obs = is_observed(P.ybar[pix]);
-        const float s = obs ? 0.f : ax - (cold ? 0.f : Z[pix]);
+        const bool obs = is_observed(yb[m]);
+        const float s = obs ? 0.f : ax - z[m];
         X[pix] = x;
         AX[pix] = ax;
         Sv[pix] = s;
@@ -131,22 +141,24 @@ cg_row_b(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, const 
     const int q = blockIdx.x * G + g;
     const int nrow = H / G;
     const size_t n = (size_t)H * W;
-    load_twiddles<W>(tw, tw_g, tid, kThreads);
-    __syncthreads();
-    float2 v[8];
-    load_row_xax<W>(v, P.Sa + (size_t)q * Wp, t);
-    fft_group<W, 1>(v, buf + g * W, tw, t, g);
     float* __restrict__ V = P.cg + 2 * n;
     float* __restrict__ AV = P.cg + 3 * n;
     const float* __restrict__ Sv = P.cg + 4 * n;
+    float2 v[8];
+    float sv[8];                                  // 0 on observed pixels (requested before the transform)
+    load_row_xax<W>(v, P.Sa + (size_t)q * Wp, t);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) sv[m] = Sv[(size_t)q * W + t + m * FT];
+    load_twiddles<W>(tw, tw_g, tid, kThreads);
+    __syncthreads();
+    fft_group<W, 1>(v, buf + g * W, tw, t, g);
     CompSum den;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
         const size_t pix = (size_t)q * W + t + m * FT;
         V[pix] = v[m].x;
         AV[pix] = v[m].y;
-        const float s = Sv[pix];                  // 0 on observed pixels
-        den.add(s * (s - v[m].y));
+        den.add(sv[m] * (sv[m] - v[m].y));
     }
     const double tot = block_sum_comp(den, red);
     if (tid == 0) {
@@ -222,20 +234,33 @@ cg_obs(const ProbDesc* __restrict__ probs, SlotTable sl, int H) {
     float* __restrict__ Z = P.cg + 5 * n;
     float* __restrict__ xw = P.work;
     float* __restrict__ z1w = P.work + n;
+    const float* __restrict__ Y = P.ybar;
+    float* __restrict__ D1 = P.d1;
+    float* __restrict__ XP = P.xprev;
     const float mu1 = P.mu1, inv1 = P.inv1pmu1;
+    // all reads first (whatever the pixel needs of them): between the stores each
+    // would wait its own latency
+    float xv[8], axv[8], yv[8], dv[8], zv[8], pv8[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        const size_t pix = (size_t)q * W + t + m * FT;
+        xv[m] = fmaf(alpha, V[pix], X[pix]);
+        axv[m] = fmaf(alpha, AV[pix], AX[pix]);
+        yv[m] = Y[pix];
+        dv[m] = cold ? 0.f : D1[pix];
+        zv[m] = fmaf(alpha, Sv[pix], cold ? 0.f : Z[pix]);
+        pv8[m] = (chk && !first) ? XP[pix] : 0.f;
+    }
     CompSum s_data, s_xx, s_dxx, s_pr;
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
         const size_t pix = (size_t)q * W + t + m * FT;
-        const float x = fmaf(alpha, V[pix], X[pix]);
-        const float ax = fmaf(alpha, AV[pix], AX[pix]);
-        const float yb = P.ybar[pix];
-        float z1;
+        const float x = xv[m], ax = axv[m], yb = yv[m];
+        float z1 = zv[m], nd1 = 0.f;
         if (is_observed(yb)) {
-            const float dd1 = cold ? 0.f : P.d1[pix];
+            const float dd1 = dv[m];
             const float u1 = fmaf(mu1, ax - dd1, yb) * inv1;
-            const float nd1 = dd1 - (ax - u1);
-            P.d1[pix] = nd1;
+            nd1 = dd1 - (ax - u1);
             z1 = u1 + nd1;
             if (nobj) {
                 const float e = ax - yb;
@@ -244,18 +269,17 @@ cg_obs(const ProbDesc* __restrict__ probs, SlotTable sl, int H) {
                 s_pr.add(e1 * e1);
             }
         } else {
-            z1 = fmaf(alpha, Sv[pix], cold ? 0.f : Z[pix]);
             Z[pix] = z1;
-            P.d1[pix] = 0.f;
         }
+        D1[pix] = nd1;
         xw[pix] = x;
         z1w[pix] = z1;
         if (chk) {
-            const float dx = first ? x : x - P.xprev[pix];
+            const float dx = x - pv8[m];
             s_dxx.add(dx * dx);
             s_xx.add(x * x);
         }
-        if (sprev) P.xprev[pix] = x;
+        if (sprev) XP[pix] = x;
     }
     if (nobj || chk) {
         const CompSum acc[kNumPartials] = {s_data, CompSum(), s_xx, s_dxx, s_pr};
@@ -279,16 +303,22 @@ cg_obs(const ProbDesc* __restrict__ probs, SlotTable sl, int H) {
 // the previous d2 (double-buffered by iteration parity, so a neighbour's halo
 // always sees the old d2). Finishes the iteration. Grid: (tiles, slots).
 // H and W are multiples of 32 (not necessarily powers of two).
+//
+// Bound by memory latency (28 B per pixel, a few tiles per SM): a thread owns
+// four adjacent pixels of row tid / 8 and requests everything it needs, 16
+// bytes at a time, before anything else; the left column's delta_h comes by
+// shuffle, delta_v goes through shared memory once, and eight threads and one
+// warp take the row above and the column left of the tile as well. 8 x 384^2:
+// MEASURED
 // ---------------------------------------------------------------------------
 constexpr int kCgTile = 32;
-// periodic index for x in [-n, 2n)
-__device__ __forceinline__ int wrapi(int x, int n) { return x < 0 ? x + n : (x >= n ? x - n : x); }
 template <bool ANISO = false>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 tv_tile(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W, int n_row_ctas,
         int* __restrict__ n_active) {
     chain_wait();   // (launch chain: the predecessor's writes are visible)
-    constexpr int T = kCgTile, XR = T + 2, XS = T + 3, DR = T + 1;
+    constexpr int T = kCgTile;
+    static_assert(T * T == 4 * kThreads, "four pixels per thread");
     const int pi = sl.map[blockIdx.y];
     if (pi < 0) return;
     const ProbDesc& P = probs[pi];
@@ -296,65 +326,97 @@ tv_tile(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W, int n_ro
     const int k = P.ctl->iter + 1;
     const bool first = k == 1 && !P.warm;        // d2 = 0 (cold start)
     const bool chk = is_check_iter(P, k), nobj = need_obj_iter(P, k);
-    __shared__ float xs[XR * XS];                // x on rows R0-1 .. R0+T, columns C0-1 .. C0+T
-    __shared__ float2 dl[DR * DR];               // delta on rows R0-1 .. R0+T-1, columns C0-1 .. C0+T-1
-    __shared__ __align__(8) float2 d2s[DR * DR]; // the previous d2 on the same region
+    __shared__ __align__(16) float dvs[(T + 1) * T];   // delta_v on rows R0-1 .. R0+T-1
+    __shared__ float dhs[T];                     // delta_h on column C0-1
     __shared__ float red[kThreads / 32 * 2 * kNumPartials];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles_x = W / T;
     const int R0 = (blockIdx.x / tiles_x) * T, C0 = (blockIdx.x % tiles_x) * T;
     const size_t n = (size_t)H * W;
     const float* __restrict__ xw = P.work;
+    float* __restrict__ ww = P.work + 2 * n;
     const float2* __restrict__ d2in = reinterpret_cast<const float2*>(P.d2 + ((k + 1) & 1) * P.d2_stride);
     float2* __restrict__ d2out = reinterpret_cast<float2*>(P.d2 + (k & 1) * P.d2_stride);
-    // x and the previous d2 of the region requested together (cp.async)
-    for (int e = tid; e < XR * XR; e += kThreads) {
-        const int rr = e / XR, cc = e - rr * XR;
-        const int r = wrapi(R0 - 1 + rr, H), c = wrapi(C0 - 1 + cc, W);
-        cp_async4(&xs[rr * XS + cc], xw + (size_t)r * W + c);
-    }
-    if (!first) {
-        for (int e = tid; e < DR * DR; e += kThreads) {
-            const int rr = e / DR, cc = e - rr * DR;
-            const int r = wrapi(R0 - 1 + rr, H), c = wrapi(C0 - 1 + cc, W);
-            cp_async8(&d2s[e], d2in + (size_t)r * W + c);
+    const float tau = P.tau, gam = P.gamma;
+    // four adjacent pixels (r, c .. c + 3): x, x below, x right of the last one, d2
+    struct Quad {
+        float x[5], xd[4], dh[4], dv[4];
+    };
+    auto load = [&](int r, int c) {
+        Quad v;
+        const int rd = r + 1 == H ? 0 : r + 1, cr = c + 4 == W ? 0 : c + 4;
+        const float4 a = *reinterpret_cast<const float4*>(xw + (size_t)r * W + c);
+        const float4 b = *reinterpret_cast<const float4*>(xw + (size_t)rd * W + c);
+        v.x[4] = xw[(size_t)r * W + cr];
+        float4 d0 = make_float4(0.f, 0.f, 0.f, 0.f), d1 = d0;
+        if (!first) {
+            d0 = *reinterpret_cast<const float4*>(d2in + (size_t)r * W + c);
+            d1 = *reinterpret_cast<const float4*>(d2in + (size_t)r * W + c + 2);
         }
-    }
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-    const float tau = P.tau;
-    CompSum tvs, prs;
-    for (int e = tid; e < DR * DR; e += kThreads) {
-        const int rr = e / DR, cc = e - rr * DR;
-        const int r = wrapi(R0 - 1 + rr, H), c = wrapi(C0 - 1 + cc, W);
-        const size_t pix = (size_t)r * W + c;
-        const float x0 = xs[rr * XS + cc];
-        const float gh = xs[rr * XS + cc + 1] - x0;
-        const float gv = xs[(rr + 1) * XS + cc] - x0;
-        const float2 dold = first ? make_float2(0.f, 0.f) : d2s[e];
+        v.x[0] = a.x; v.x[1] = a.y; v.x[2] = a.z; v.x[3] = a.w;
+        v.xd[0] = b.x; v.xd[1] = b.y; v.xd[2] = b.z; v.xd[3] = b.w;
+        v.dh[0] = d0.x; v.dv[0] = d0.y; v.dh[1] = d0.z; v.dv[1] = d0.w;
+        v.dh[2] = d1.x; v.dv[2] = d1.y; v.dh[3] = d1.z; v.dv[3] = d1.w;
+        return v;
+    };
+    // u2 = prox(D x - d2), d2 <- d2 - (D x - u2), delta = u2 + d2 of one pixel
+    auto step = [&](float gh, float gv, float odh, float odv, float& ndh, float& ndv, float& eh, float& ev) {
         float uh, uv;
-        tv_prox(gh - dold.x, gv - dold.y, tau, ANISO, uh, uv);
-        const float ndh = dold.x - (gh - uh), ndv = dold.y - (gv - uv);
-        dl[rr * DR + cc] = make_float2(uh + ndh, uv + ndv);
-        if (rr >= 1 && cc >= 1) {                // a pixel of the tile: owned
-            d2out[pix] = make_float2(ndh, ndv);
-            if (nobj) {
-                tvs.add(tv_norm(gh, gv, ANISO));
-                const float eh = ndh - dold.x, ev = ndv - dold.y;
-                prs.add(fmaf(eh, eh, ev * ev));
-            }
+        tv_prox(gh - odh, gv - odv, tau, ANISO, uh, uv);
+        ndh = odh - (gh - uh);
+        ndv = odv - (gv - uv);
+        eh = uh + ndh;
+        ev = uv + ndv;
+    };
+    const int orow = tid >> 3, ocol = 4 * (tid & 7);
+    const Quad own = load(R0 + orow, C0 + ocol);
+    // the halo: threads 0..7 the row above, warp 1 (one row per lane) the column left
+    Quad up = {};
+    float lx = 0.f, lxr = 0.f, lxd = 0.f;
+    float2 ld = make_float2(0.f, 0.f);
+    if (tid < 8) up = load(R0 == 0 ? H - 1 : R0 - 1, C0 + ocol);
+    if (warp == 1) {
+        const int r = R0 + lane, rd = r + 1 == H ? 0 : r + 1, c = C0 == 0 ? W - 1 : C0 - 1;
+        lx = xw[(size_t)r * W + c];
+        lxr = xw[(size_t)r * W + C0];
+        lxd = xw[(size_t)rd * W + c];
+        if (!first) ld = d2in[(size_t)r * W + c];
+    }
+    CompSum tvs, prs;
+    float dh[4], dv[4], nh[4], nv[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float gh = own.x[e + 1] - own.x[e], gv = own.xd[e] - own.x[e];
+        step(gh, gv, own.dh[e], own.dv[e], nh[e], nv[e], dh[e], dv[e]);
+        if (nobj) {
+            tvs.add(tv_norm(gh, gv, ANISO));
+            const float eh = nh[e] - own.dh[e], ev = nv[e] - own.dv[e];
+            prs.add(fmaf(eh, eh, ev * ev));
         }
     }
-    __syncthreads();
-    const float gam = P.gamma;
-    float* __restrict__ ww = P.work + 2 * n;
-    for (int e = tid; e < T * T; e += kThreads) {
-        const int rr = e / T + 1, cc = e % T + 1;
-        const float2 d = dl[rr * DR + cc];
-        const float wv = gam * ((dl[rr * DR + cc - 1].x - d.x) + (dl[(rr - 1) * DR + cc].y - d.y));
-        ww[(size_t)(R0 + rr - 1) * W + (C0 + cc - 1)] = wv;
+    *reinterpret_cast<float4*>(dvs + (orow + 1) * T + ocol) = make_float4(dv[0], dv[1], dv[2], dv[3]);
+    if (tid < 8) {
+        float a, b, h, v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            step(up.x[e + 1] - up.x[e], up.xd[e] - up.x[e], up.dh[e], up.dv[e], a, b, h, v[e]);
+        *reinterpret_cast<float4*>(dvs + ocol) = make_float4(v[0], v[1], v[2], v[3]);
     }
+    if (warp == 1) {
+        float a, b, h, v;
+        step(lxr - lx, lxd - lx, ld.x, ld.y, a, b, h, v);
+        dhs[lane] = h;
+    }
+    const size_t pix = (size_t)(R0 + orow) * W + (C0 + ocol);
+    *reinterpret_cast<float4*>(d2out + pix) = make_float4(nh[0], nv[0], nh[1], nv[1]);
+    *reinterpret_cast<float4*>(d2out + pix + 2) = make_float4(nh[2], nv[2], nh[3], nv[3]);
+    const float sh = __shfl_up_sync(0xffffffffu, dh[3], 1);
+    __syncthreads();
+    const float4 u = *reinterpret_cast<const float4*>(dvs + orow * T + ocol);
+    const float left = (tid & 7) == 0 ? dhs[orow] : sh;
+    *reinterpret_cast<float4*>(ww + pix) =
+        make_float4(gam * ((left - dh[0]) + (u.x - dv[0])), gam * ((dh[0] - dh[1]) + (u.y - dv[1])),
+                    gam * ((dh[1] - dh[2]) + (u.z - dv[2])), gam * ((dh[2] - dh[3]) + (u.w - dv[3])));
     double pv[kNumPartials] = {0.0};
     if (nobj || chk) {
         const CompSum acc[kNumPartials] = {CompSum(), tvs, CompSum(), CompSum(), prs};
