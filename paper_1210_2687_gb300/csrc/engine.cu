@@ -131,7 +131,17 @@ struct DeviceCtx {
 // independent graph branches, so one lane's column phase (transform-bound)
 // can share the GPU with the other lane's row phase (memory-bound).
 constexpr int kMaxLanes = 4;
-constexpr int kDefaultLanes = 2;
+// Lanes of an untuned class. Two lanes pay once each lane's launches fill the
+// GPU by themselves; below that they only halve launches that are short of
+// CTAs and double their number. Measured, us per problem and iteration, one
+// lane / two: TV 512^2 x 4 9.07 / 10.75, x 8 6.63 / 7.06, x 16 6.11 / 5.76;
+// 256^2 x 8 2.94 / 3.31, x 64 1.84 / 1.74; 1024^2 x 2 33.1 / 33.2, x 4 30.5 /
+// 29.1; frame 512^2 x 4 21.2 / 22.1, x 16 17.9 / 16.7; mixed radix 384^2 x 4
+// 9.66 / 11.73, 768 x 640 x 4 22.1 / 22.2, 384^2 x 16 5.96 / 5.86;
+// Reeves-Sorel 256^2 x 8 6.57 / 8.11, x 16 4.90 / 5.23. The lines cross
+// between 2 and 2.4 Mpixel in flight.
+constexpr long long kOneLanePixels = 1ll << 21;
+inline int default_lanes(int H, int W, int slots) { return (long long)H * W * slots <= kOneLanePixels ? 1 : 2; }
 struct Lanes {
     int n = 1;
     int off[kMaxLanes] = {}, cnt[kMaxLanes] = {}, soff[kMaxLanes] = {}, slots[kMaxLanes] = {};
@@ -313,7 +323,13 @@ int gen_twiddles(DeviceCtx* c, int N, const float2** out) {
 // ---- tiling choices -----------------------------------------------------
 // Defaults are entry 0 of the compiled candidate lists (variants.cuh); the
 // tuning table overrides them per (device, H, W, regulariser, levels).
-constexpr int kDefaultSlotCtas = 2400;
+// A slot costs one table word, so the target is high: launches that hold more
+// problems leave a shorter last wave, and fewer problems queue up to run
+// alone at the end. Measured against 2400 (us per problem and iteration): TV
+// 512^2 x 64 5.08 -> 5.03, x 160 4.85 -> 4.71, 256^2 x 300 1.82 -> 1.76,
+// 1024^2 x 16 24.6 -> 24.1; frame 512^2 x 64 15.3 -> 14.7, 1024^2 x 24 64.2 ->
+// 57.7. 19200 gives no more (4.65, 1.77, 24.2; 14.5, 57.7).
+constexpr int kDefaultSlotCtas = 9600;
 
 int col_block(int H) {
     const ColVariant* v = nullptr;
@@ -325,8 +341,7 @@ int row_strip_tv(int W) {
 }
 
 // launch slots of a group: enough problems in flight that a row-side launch
-// has about `slot_ctas` CTAs (default some eight waves of two CTAs per SM on
-// 152 SMs)
+// has about `slot_ctas` CTAs
 int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count) {
     const int per = tv ? H / R : haar_num_tiles(H, W);
     const int target = slot_ctas > 0 ? slot_ctas : kDefaultSlotCtas;
@@ -1260,7 +1275,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
         // (as is a class that runs in teams)
         team = team && g.tv && !g.gen && g.row_v == 0 && g.nslots == g.count &&
                use_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, g.count);
-        g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : kDefaultLanes, g.count, g.nslots}));
+        g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : default_lanes(g.H, g.W, g.nslots), g.count, g.nslots}));
         for (int l = 0, o = g.off, so = soff; l < g.L.n; ++l) {
             g.L.off[l] = o;
             g.L.cnt[l] = l + 1 < g.L.n ? g.count / g.L.n : g.off + g.count - o;
