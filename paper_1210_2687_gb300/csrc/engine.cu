@@ -321,7 +321,7 @@ int gen_twiddles(DeviceCtx* c, int N, const float2** out) {
 }
 
 // ---- tiling choices -----------------------------------------------------
-// Defaults are entry 0 of the compiled candidate lists (variants.cuh); the
+// Defaults are those of the compiled candidate lists (variants.cuh); the
 // tuning table overrides them per (device, H, W, regulariser, levels).
 // A slot costs one table word, so the target is high: launches that hold more
 // problems leave a shorter last wave, and fewer problems queue up to run
@@ -337,7 +337,7 @@ int col_block(int H) {
 }
 int row_strip_tv(int W) {
     const RowVariant* v = nullptr;
-    return tv_row_variants(W, &v) > 0 ? v[0].R : 0;
+    return tv_row_variants(W, &v) > 0 ? v[tv_row_default(W)].R : 0;
 }
 
 // launch slots of a group: enough problems in flight that a row-side launch
@@ -353,7 +353,7 @@ int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count) {
 using TuneKey = std::tuple<int, int, int, int, int>;   // device, H, W, reg, levels
 std::map<TuneKey, admm_tuning_t> g_tuning;            // under g_mutex
 
-// the configuration a new plan of this class gets (entry 0 when untuned)
+// the configuration a new plan of this class gets (the default when untuned)
 admm_tuning_t lookup_tuning(int dev, int H, int W, int reg, int levels) {
     auto it = g_tuning.find(TuneKey(dev, H, W, reg, levels));
     if (it != g_tuning.end()) return it->second;
@@ -362,6 +362,7 @@ admm_tuning_t lookup_tuning(int dev, int H, int W, int reg, int levels) {
     t.W = W;
     t.reg = reg;
     t.haar_levels = levels;
+    if (reg == ADMM_REG_TV) t.row_variant = tv_row_default(W);
     return t;
 }
 
@@ -403,7 +404,7 @@ cudaError_t launch_row_tv(int W, const ProbDesc* d, SlotTable sl, int count, int
                           int* n_active, cudaStream_t s) {
     const RowVariant* v = nullptr;
     if (tv_row_variants(W, &v) == 0) return cudaErrorInvalidValue;
-    return v[0].fn(d, sl, count, H, Wp, tw, n_active, s);
+    return v[tv_row_default(W)].fn(d, sl, count, H, Wp, tw, n_active, s);
 }
 
 template <int W>

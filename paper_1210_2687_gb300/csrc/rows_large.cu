@@ -1,6 +1,6 @@
 // rows_large.cu -- compiled TV row-phase configurations for W = 1024, 2048
-// (rows per strip, walk rows in flight, threads per CTA); entry 0 is the
-// default of each width.
+// (rows per strip, walk rows in flight, threads per CTA); the default is
+// tv_row_default of each width.
 #include "variants.cuh"
 
 namespace admm {

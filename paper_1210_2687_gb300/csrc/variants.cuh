@@ -4,7 +4,7 @@
 // Every side length has a short list of compiled configurations of the TV
 // row phase (rows per strip R, walk rows in flight D, threads per CTA NT) and
 // of the column phase (columns per CTA CB); entry 0 of each list is the
-// default. The autotuner (admm_deconv_autotune) times the combinations on the
+// default, but for rows of 2048 (tv_row_default). The autotuner (admm_deconv_autotune) times the combinations on the
 // device and records the fastest per (device, H, W, regulariser, levels);
 // plans created afterwards use it. The instantiations are spread over
 // several translation units (rows_small.cu, rows_512.cu, rows_large.cu,
@@ -36,6 +36,13 @@ struct ColVariant {
 // candidates for one side length (entry 0 = default); returns their number,
 // 0 for an unsupported side
 int tv_row_variants(int W, const RowVariant** out);
+// the TV row configuration of an untuned class. At W = 2048 a strip of two
+// rows does 2x the inverse transforms that its rows need (four rows: 1.5x),
+// but it holds half the shared memory, so that twice the CTAs hide the walk's
+// latencies: 2048^2 x 1 152.8 -> 132.8 us per iteration (both phases), x 2
+// 130.4 -> 116.8, x 4 120.2 -> 115.3; 1024 x 2048 x 2 69.6 -> 64.3. Elsewhere
+// entry 0 is the fastest of its list for one image and within 5 % for many.
+inline int tv_row_default(int W) { return W == 2048 ? 2 : 0; }
 int col_variants(int H, const ColVariant** out);
 
 // per translation unit
