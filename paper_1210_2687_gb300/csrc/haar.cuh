@@ -455,58 +455,69 @@ haar_analysis(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W, in
 // bands at (r - {0, s}, c - {0, s}), so the tile needs zeta2 of level j on
 // [-(2^{j+1} - 1), T)^2 and the low-low band on [-(2^L - 1), T)^2.
 // Runs after haar_analysis has finished the iteration (ctl->iter = k).
+//
+// Bound by shared memory: 13 bands are read with halos, every element four
+// times by the formula. The rows adjoint (lo, hi) of a column is formed once
+// and handed to the column s to the right by shuffle (which halves the
+// reads), every level's arrays are only as wide as its own halo (36, 36, 40,
+// 48 columns: rows start on distinct banks, and 15 % less arrives by TMA) and
+// a level's output replaces its input through registers, so that four CTAs
+// fit on an SM. 2048^2 (4 levels): 70.3 -> 50.6 us.
 // ---------------------------------------------------------------------------
 template <int L>
 struct HaarSynCfg {
     static constexpr int T = kHaarTile;
     static constexpr int HALO = (1 << L) - 1;
-    static_assert(HALO < 16, "halo fits the 16-column margin");
-    // every array spans the columns [-16, T) (16-byte copies from a tile
-    // origin that is a multiple of 32 columns) and the rows it needs
-    static constexpr int XS = T + 16;              // row stride of every array
-    static constexpr int AR = T + HALO;            // approximation arrays: rows [-HALO, T)
-    __host__ __device__ static constexpr int band_rows(int lvl) { return T + 2 * (1 << lvl) - 1; }
-    // two band slots, each sized for the coarsest level: level j lives in slot
-    // j % 2, and the bands of level j - 1 are requested into the other slot as
-    // soon as level j + 1 has released it. Array sizes are rounded to 32
-    // floats, so that the TMA destinations (the low-low array and the two
-    // slots) start on 128-byte boundaries; two mbarriers follow.
-    static constexpr int ARS = (AR * XS + 31) / 32 * 32;
-    static constexpr int SLOT = (3 * band_rows(L - 1) * XS + 31) / 32 * 32;
-    static constexpr size_t BAR_OFF = (size_t)(2 * ARS + 2 * SLOT) * sizeof(float);
+    static_assert(HALO < 16, "halo fits four groups of four columns");
+    // the arrays of a level span the rows [-rows_halo, T) and the columns
+    // [-4 groups, T): groups of four columns that hold its 2^{lvl+1} - 1 halo
+    // columns (16-byte copies from a tile origin that is a multiple of 32)
+    __host__ __device__ static constexpr int groups(int lvl) { return (2 * (1 << lvl) - 1 + 3) / 4; }
+    __host__ __device__ static constexpr int rows(int lvl) { return T + 2 * (1 << lvl) - 1; }
+    __host__ __device__ static constexpr int cols(int lvl) { return T + 4 * groups(lvl); }
+    __host__ __device__ static constexpr int pad32(int n) { return (n + 31) / 32 * 32; }
+    // two band slots, level j in slot j % 2, each sized for the coarsest level
+    // it holds; array sizes are rounded to 32 floats, so that the TMA
+    // destinations (the low-low array and the two slots) start on 128-byte
+    // boundaries; two mbarriers follow
+    __host__ __device__ static constexpr int slot_floats(int p) {
+        const int top = ((L - 1) & 1) == p ? L - 1 : L - 2;
+        return top < 0 ? 0 : pad32(3 * rows(top) * cols(top));
+    }
+    static constexpr int ARS = pad32(rows(L - 1) * cols(L - 1));
+    __host__ __device__ static constexpr int slot_off(int lvl) { return ARS + ((lvl & 1) ? slot_floats(0) : 0); }
+    static constexpr size_t BAR_OFF = (size_t)(ARS + slot_floats(0) + slot_floats(1)) * sizeof(float);
     static constexpr size_t SMEM = BAR_OFF + 2 * sizeof(unsigned long long);
 };
 
 // Host: the L + 1 tensor maps the synthesis tile loads its halo boxes with,
 // over both d2 buffers of a problem viewed as a 4-D tensor (W columns, H rows,
-// 3 L + 1 bands, 2 buffers; FP32): map 0 the low-low band's box (T + 16
-// columns x T + 2^L - 1 rows x 1 band), map 1 + j level j's three bands
-// (T + 16 columns x T + 2^{j+1} - 1 rows x 3 bands). `enc` is the driver's
-// cuTensorMapEncodeTiled; false if a map cannot be encoded.
+// 3 L + 1 bands, 2 buffers; FP32): map 0 the low-low band's box (the columns
+// and rows of the coarsest level, 1 band), map 1 + j level j's three bands.
+// `enc` is the driver's cuTensorMapEncodeTiled; false if a map cannot be
+// encoded.
 template <typename Enc, typename Map>
 bool haar_synthesis_maps(Enc enc, Map* maps, float* d2, int H, int W, int levels) {
+    using C = HaarSynCfg<1>;                      // (rows and columns of a level do not depend on L)
     const int nb = 3 * levels + 1;
     const uint64_t n = (uint64_t)H * W;
     const uint64_t dims[4] = {(uint64_t)W, (uint64_t)H, (uint64_t)nb, 2};
     const uint64_t strides[3] = {(uint64_t)W * 4, n * 4, (uint64_t)nb * n * 4};
     const uint32_t es[4] = {1, 1, 1, 1};
     for (int i = 0; i <= levels; ++i) {
-        const uint32_t rows = i == 0 ? (uint32_t)(kHaarTile + (1 << levels) - 1)
-                                     : (uint32_t)(kHaarTile + 2 * (1 << (i - 1)) - 1);
-        const uint32_t box[4] = {(uint32_t)(kHaarTile + 16), rows, i == 0 ? 1u : 3u, 1u};
+        const int lvl = i == 0 ? levels - 1 : i - 1;
+        const uint32_t box[4] = {(uint32_t)C::cols(lvl), (uint32_t)C::rows(lvl), i == 0 ? 1u : 3u, 1u};
         if (!enc(&maps[i], d2, dims, strides, box, es)) return false;
     }
     return true;
 }
 
 template <int L>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 4)
 haar_synthesis(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W) {
     chain_wait();   // (launch chain: the predecessor's writes are visible)
     using C = HaarSynCfg<L>;
-    constexpr int T = C::T, HALO = C::HALO, XS = C::XS, AR = C::AR;
-    constexpr int CH = XS / 4;                     // 16-byte chunks per array row
-    constexpr int NWARP = kThreads / 32;
+    constexpr int T = C::T;
     const int pi = sl.map[blockIdx.y];
     if (pi < 0) return;
     const ProbDesc& P = probs[pi];
@@ -515,8 +526,6 @@ haar_synthesis(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W) {
     extern __shared__ __align__(128) float syn_sm[];
     float* sm = syn_sm;
     float* At = sm;
-    float* Ao = sm + C::ARS;
-    float* Z = sm + 2 * C::ARS;
     unsigned long long* bars = reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(sm) + C::BAR_OFF);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tiles_x = W / T;
@@ -533,31 +542,31 @@ haar_synthesis(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W) {
     const bool tma = P.zmap != nullptr && R0 > 0 && C0 > 0 && (smem_u32(sm) & 127u) == 0;
     const char* zmaps = static_cast<const char*>(P.zmap);
     auto tma_request = [&](int lvl) {
-        const int BO = 2 * (1 << lvl) - 1;
+        const int x = C0 - 4 * C::groups(lvl), y = R0 - (C::rows(lvl) - T);
         const uint32_t bar = smem_u32(&bars[lvl & 1]);
-        const uint32_t bytes = 3u * (uint32_t)((T + BO) * XS) * 4u + (lvl == L - 1 ? (uint32_t)(AR * XS) * 4u : 0u);
-        mbar_expect_tx(bar, bytes);
-        if (lvl == L - 1) tma_load_4d(At, zmaps, C0 - 16, R0 - HALO, 3 * L, zb, bar);
-        tma_load_4d(Z + (lvl & 1) * C::SLOT, zmaps + 128 * (1 + lvl), C0 - 16, R0 - BO, 3 * lvl, zb, bar);
+        const uint32_t plane = (uint32_t)(C::rows(lvl) * C::cols(lvl)) * 4u;
+        mbar_expect_tx(bar, lvl == L - 1 ? 4u * plane : 3u * plane);
+        if (lvl == L - 1) tma_load_4d(At, zmaps, x, y, 3 * L, zb, bar);
+        tma_load_4d(sm + C::slot_off(lvl), zmaps + 128 * (1 + lvl), x, y, 3 * lvl, zb, bar);
     };
 
-    // low-low band on rows [-HALO, T) and each level's bands on rows [-BO, T),
-    // all on the columns [-16, T), one cp.async group per level (the low-low
-    // band with the coarsest). Two levels are requested at entry; each later
-    // level goes into the slot the level before last has just released, so
-    // its loads overlap the adjoint of the level in between.
-    auto request = [&](int lvl) {
-        const int BO = 2 * (1 << lvl) - 1, BR = T + BO;
-        float* Zl = Z + (lvl & 1) * C::SLOT;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float* band = zeta + (size_t)(3 * lvl + j) * n;
-            for (int e = tid; e < BR * CH; e += kThreads) {
-                const int rr = e / CH, ch = e - rr * CH;
-                cp_async16(Zl + (j * BR + rr) * XS + 4 * ch,
-                           band + (size_t)hwrap(R0 + rr - BO, H) * W + hwrap(C0 - 16 + 4 * ch, W));
-            }
+    // one band on the rows and columns of level lvl into `dst`
+    auto copy_band = [&](float* dst, const float* band, int lvl) {
+        const int CH = C::cols(lvl) / 4, BO = C::rows(lvl) - T;
+        for (int e = tid; e < C::rows(lvl) * CH; e += kThreads) {
+            const int rr = e / CH, ch = e - rr * CH;
+            cp_async16(dst + 4 * e,
+                       band + (size_t)hwrap(R0 + rr - BO, H) * W + hwrap(C0 - 4 * C::groups(lvl) + 4 * ch, W));
         }
+    };
+    // each level's bands, one cp.async group per level (the low-low band with
+    // the coarsest). Two levels are requested at entry; each later level goes
+    // into the slot that the level before last has just released, so its
+    // loads overlap the adjoint of the level in between.
+    auto request = [&](int lvl) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            copy_band(sm + C::slot_off(lvl) + j * C::rows(lvl) * C::cols(lvl), zeta + (size_t)(3 * lvl + j) * n, lvl);
         cp_async_commit();
     };
     if (tma) {
@@ -568,119 +577,118 @@ haar_synthesis(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int W) {
             tma_request(L - 1);
             if (L >= 2) tma_request(L - 2);
         }
-        __syncthreads();             // the barriers are initialised before anyone waits on them
     } else {
-        const float* band = zeta + (size_t)(3 * L) * n;
-        for (int e = tid; e < AR * CH; e += kThreads) {
-            const int rr = e / CH, ch = e - rr * CH;
-            cp_async16(At + rr * XS + 4 * ch,
-                       band + (size_t)hwrap(R0 + rr - HALO, H) * W + hwrap(C0 - 16 + 4 * ch, W));
-        }
+        copy_band(At, zeta + (size_t)(3 * L) * n, L - 1);
         request(L - 1);
         if (L >= 2) request(L - 2);
     }
+    const float gam = P.gamma;
+    float* __restrict__ ww = P.work + 2 * n;
+    __syncthreads();                 // the barriers are initialised before anyone waits on them
 
+    // A warp takes four rows, eight lanes per row: lane gq owns the columns
+    // 4 gq .. + 3, and of the halo the group 4 (gq - 8), where the level has it.
+    static_assert(T == 32 && kThreads == 256, "eight column groups per row, 32 rows per pass");
+    const int rr = lane >> 3, gq = lane & 7;
 #pragma unroll
     for (int lvl = L - 1; lvl >= 0; --lvl) {
-        // this level's bands have landed (at the first level the next one may
-        // still be in flight; later, the next level is requested only below)
+        // this level's bands have landed (the next level's may still be in flight)
         if (tma) {
             // slot lvl % 2 completes its ((L - 1 - lvl) / 2)-th phase with this level
             const uint32_t parity = (uint32_t)((L - 1 - lvl) >> 1) & 1u;
             if (!mbar_wait_bounded(smem_u32(&bars[lvl & 1]), parity) && tid == 0)
                 atomicExch(&P.ctl->status, kStatusTimeout);
-        } else if (lvl == L - 1 && L >= 2) {
-            cp_async_wait<1>();
         } else {
-            cp_async_wait<0>();
+            if (lvl >= 1) cp_async_wait<1>();
+            else cp_async_wait<0>();
+            __syncthreads();         // ... for every thread
         }
-        __syncthreads();             // ... for every thread; level lvl + 1 is done and its slot free
-        if (lvl <= L - 2 && lvl >= 1) {
+        constexpr int kMaxPass = 2;
+        const int s = 1 << lvl;
+        const int D = T + s - 1;                       // output rows [-(s-1), T)
+        const int BO = C::rows(lvl) - T, XS = C::cols(lvl), NH = C::groups(lvl);
+        const int NO = lvl > 0 ? C::groups(lvl - 1) : 0;   // halo groups of the output
+        const int rs = s * XS;
+        const float* Z0 = sm + C::slot_off(lvl);
+        const float* Z1 = Z0 + C::rows(lvl) * XS;
+        const float* Z2 = Z1 + C::rows(lvl) * XS;
+        // lo = (At + At') + (Z1 - Z1'), hi = (Z0 + Z0') + (Z2 - Z2') of four
+        // columns, ' the row s above
+        auto rows_adjoint = [&](int i, float (&lo)[4], float (&hi)[4]) {
+            const float4 t0 = *reinterpret_cast<const float4*>(At + i), t1 = *reinterpret_cast<const float4*>(At + i - rs);
+            const float4 u0 = *reinterpret_cast<const float4*>(Z1 + i), u1 = *reinterpret_cast<const float4*>(Z1 + i - rs);
+            const float4 g0 = *reinterpret_cast<const float4*>(Z0 + i), g1 = *reinterpret_cast<const float4*>(Z0 + i - rs);
+            const float4 h0 = *reinterpret_cast<const float4*>(Z2 + i), h1 = *reinterpret_cast<const float4*>(Z2 + i - rs);
+            lo[0] = (t0.x + t1.x) + (u0.x - u1.x); hi[0] = (g0.x + g1.x) + (h0.x - h1.x);
+            lo[1] = (t0.y + t1.y) + (u0.y - u1.y); hi[1] = (g0.y + g1.y) + (h0.y - h1.y);
+            lo[2] = (t0.z + t1.z) + (u0.z - u1.z); hi[2] = (g0.z + g1.z) + (h0.z - h1.z);
+            lo[3] = (t0.w + t1.w) + (u0.w - u1.w); hi[3] = (g0.w + g1.w) + (h0.w - h1.w);
+        };
+        // lanes whose groups lie s columns to the left: one lane (s <= 4) or two
+        const int step = s > 4 ? 2 : 1;
+        const int left = (lane & 24) | ((gq - step) & 7);
+        float out[kMaxPass][4], hout[kMaxPass][4];
+#pragma unroll
+        for (int p = 0; p < kMaxPass; ++p) {
+            const int row = 32 * p + 4 * warp + rr;    // from the first output row
+            if (32 * p + 4 * warp >= D) continue;      // (the whole warp)
+            const int r = min(row, D - 1) - (s - 1);   // lanes past the last row repeat it
+            const int i0 = (r + BO) * XS + 4 * NH;
+            float lo[4], hi[4], hlo[4] = {0.f, 0.f, 0.f, 0.f}, hhi[4] = {0.f, 0.f, 0.f, 0.f};
+            rows_adjoint(i0 + 4 * gq, lo, hi);
+            if (gq >= 8 - NH) rows_adjoint(i0 + 4 * (gq - 8), hlo, hhi);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                // columns c + e - s: the lane's own, or the left lane's (around
+                // the row's start the halo group that lane holds)
+                float lol, hil, hlol, hhil;
+                if (e >= s) {
+                    lol = lo[e - s]; hil = hi[e - s]; hlol = hlo[e - s]; hhil = hhi[e - s];
+                } else {
+                    const int k = s > 4 ? e : e - s + 4;
+                    const bool wrapped = gq >= 8 - step;
+                    lol = __shfl_sync(0xffffffffu, wrapped ? hlo[k] : lo[k], left);
+                    hil = __shfl_sync(0xffffffffu, wrapped ? hhi[k] : hi[k], left);
+                    hlol = hhil = 0.f;
+                    // (s <= 2: the halo outputs that are read need only their own group)
+                    if (s >= 4) {
+                        hlol = __shfl_sync(0xffffffffu, hlo[k], left);
+                        hhil = __shfl_sync(0xffffffffu, hhi[k], left);
+                    }
+                }
+                out[p][e] = 0.25f * ((lo[e] + lol) + (hi[e] - hil));
+                hout[p][e] = 0.25f * ((hlo[e] + hlol) + (hhi[e] - hhil));
+            }
+        }
+        if (lvl == 0) {
+            // w = gamma P^T zeta2 on the tile
+            const int r = 4 * warp + rr;
+            *reinterpret_cast<float4*>(ww + (size_t)(R0 + r) * W + (C0 + 4 * gq)) =
+                make_float4(gam * out[0][0], gam * out[0][1], gam * out[0][2], gam * out[0][3]);
+            break;
+        }
+        __syncthreads();             // everyone has read this level: At and the slot are free
+        if (lvl >= 2) {
             if (!tma) {
-                request(lvl - 1);
+                request(lvl - 2);
             } else if (tid == 0) {
                 fence_proxy_async_smem();   // the slot's generic reads before the copy's writes
-                tma_request(lvl - 1);
+                tma_request(lvl - 2);
             }
         }
-        const int s = 1 << lvl;
-        const int D = T + s - 1;                       // output on [-(s-1), T)
-        const int BO = 2 * s - 1, BR = T + BO;
-        const float* Z0 = Z + (lvl & 1) * C::SLOT;
-        const float* Z1 = Z0 + BR * XS;
-        const float* Z2 = Z1 + BR * XS;
-        const int ra = s * XS, rz = s * XS;
-        // the outputs on [-(s-1), T)^2. Columns [0, T) in groups of four
-        // adjacent columns, eight groups per row, so that the eight threads of
-        // a 16-byte access phase read one 128-byte row segment: 16-byte reads of
-        // the eight input rows (At, Z0, Z1, Z2 at rows r and r - s) over columns
-        // c - s .. c + 3 and one 16-byte store. The s - 1 halo columns left of
-        // the tile one output per thread. (s, D are constants where the level
-        // loop is unrolled.)
-        static_assert(T == 32, "eight column groups per row");
-        const int nwd = s > 4 ? 3 : 2;                 // float4 words covering 4 + s columns
-        const int wb = -4 * (nwd - 1);                 // the window starts this many columns before c
-        for (int e = tid; e < D * 8; e += kThreads) {
-            const int r = (e >> 3) - (s - 1), c = 4 * (e & 7);
-            const int ia = (r + HALO) * XS + (c + 16);
-            const int iz = (r + BO) * XS + (c + 16);
-            float a0[12], a1[12], q0[12], q1[12], y0[12], y1[12], v0[12], v1[12];
+        const int XO = T + 4 * NO;                     // columns of the next level's arrays
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                if (q < nwd) {
-                    const int o = wb + 4 * q;
-                    const float4 t0 = *reinterpret_cast<const float4*>(At + ia + o);
-                    const float4 t1 = *reinterpret_cast<const float4*>(At + ia - ra + o);
-                    const float4 u0 = *reinterpret_cast<const float4*>(Z1 + iz + o);
-                    const float4 u1 = *reinterpret_cast<const float4*>(Z1 + iz - rz + o);
-                    const float4 g0 = *reinterpret_cast<const float4*>(Z0 + iz + o);
-                    const float4 g1 = *reinterpret_cast<const float4*>(Z0 + iz - rz + o);
-                    const float4 h0 = *reinterpret_cast<const float4*>(Z2 + iz + o);
-                    const float4 h1 = *reinterpret_cast<const float4*>(Z2 + iz - rz + o);
-                    a0[4 * q] = t0.x; a0[4 * q + 1] = t0.y; a0[4 * q + 2] = t0.z; a0[4 * q + 3] = t0.w;
-                    a1[4 * q] = t1.x; a1[4 * q + 1] = t1.y; a1[4 * q + 2] = t1.z; a1[4 * q + 3] = t1.w;
-                    q0[4 * q] = u0.x; q0[4 * q + 1] = u0.y; q0[4 * q + 2] = u0.z; q0[4 * q + 3] = u0.w;
-                    q1[4 * q] = u1.x; q1[4 * q + 1] = u1.y; q1[4 * q + 2] = u1.z; q1[4 * q + 3] = u1.w;
-                    y0[4 * q] = g0.x; y0[4 * q + 1] = g0.y; y0[4 * q + 2] = g0.z; y0[4 * q + 3] = g0.w;
-                    y1[4 * q] = g1.x; y1[4 * q + 1] = g1.y; y1[4 * q + 2] = g1.z; y1[4 * q + 3] = g1.w;
-                    v0[4 * q] = h0.x; v0[4 * q + 1] = h0.y; v0[4 * q + 2] = h0.z; v0[4 * q + 3] = h0.w;
-                    v1[4 * q] = h1.x; v1[4 * q + 1] = h1.y; v1[4 * q + 2] = h1.z; v1[4 * q + 3] = h1.w;
-                }
-            }
-            float out[4];
-#pragma unroll
-            for (int e4 = 0; e4 < 4; ++e4) {
-                const int kc = -wb + e4, kl = kc - s;  // window positions of columns c + e4 and c + e4 - s
-                // rows adjoint at columns c and c - s
-                const float lo_c = (a0[kc] + a1[kc]) + (q0[kc] - q1[kc]);
-                const float lo_l = (a0[kl] + a1[kl]) + (q0[kl] - q1[kl]);
-                const float hi_c = (y0[kc] + y1[kc]) + (v0[kc] - v1[kc]);
-                const float hi_l = (y0[kl] + y1[kl]) + (v0[kl] - v1[kl]);
-                out[e4] = 0.25f * ((lo_c + lo_l) + (hi_c - hi_l));
-            }
-            *reinterpret_cast<float4*>(Ao + ia) = make_float4(out[0], out[1], out[2], out[3]);
+        for (int p = 0; p < kMaxPass; ++p) {
+            const int row = 32 * p + 4 * warp + rr;
+            if (row >= D) continue;
+            const int io = row * XO + 4 * NO;
+            *reinterpret_cast<float4*>(At + io + 4 * gq) = make_float4(out[p][0], out[p][1], out[p][2], out[p][3]);
+            if (gq >= 8 - NO)
+                *reinterpret_cast<float4*>(At + io + 4 * (gq - 8)) =
+                    make_float4(hout[p][0], hout[p][1], hout[p][2], hout[p][3]);
         }
-        for (int e = tid; e < D * (s - 1); e += kThreads) {
-            const int rr = e / (s > 1 ? s - 1 : 1), cc = e - rr * (s - 1);
-            const int r = rr - (s - 1), c = cc - (s - 1);
-            const int ia = (r + HALO) * XS + (c + 16);
-            const int iz = (r + BO) * XS + (c + 16);
-            const float lo_c = (At[ia] + At[ia - ra]) + (Z1[iz] - Z1[iz - rz]);
-            const float lo_l = (At[ia - s] + At[ia - ra - s]) + (Z1[iz - s] - Z1[iz - rz - s]);
-            const float hi_c = (Z0[iz] + Z0[iz - rz]) + (Z2[iz] - Z2[iz - rz]);
-            const float hi_l = (Z0[iz - s] + Z0[iz - rz - s]) + (Z2[iz - s] - Z2[iz - rz - s]);
-            Ao[ia] = 0.25f * ((lo_c + lo_l) + (hi_c - hi_l));
-        }
-        float* tmp = At;
-        At = Ao;
-        Ao = tmp;
+        __syncthreads();             // the next level's approximation is complete
     }
-    __syncthreads();                 // the finest level is complete
-    // w = gamma P^T zeta2 on the tile
-    const float gam = P.gamma;
-    float* __restrict__ ww = P.work + 2 * n;
-    for (int r = warp; r < T; r += NWARP)
-        ww[(size_t)(R0 + r) * W + (C0 + lane)] = gam * At[(r + HALO) * XS + (lane + 16)];
 }
 
 // ---------------------------------------------------------------------------
