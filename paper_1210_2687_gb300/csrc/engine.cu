@@ -15,6 +15,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -62,7 +63,9 @@ struct admm_plan_s {
     std::vector<float> band_mu;  // one penalty per frame band (empty: mu2 for all)
     int device = 0;
     int Wc = 0, Wp = 0, cb = 0, R = 0, n_strips = 0, n_slots = 0, nb = 0, levels = 0;
-    int row_v = 0, col_v = 0, slot_ctas = 0, lanes = 0;   // launch configuration (tuning table at plan time)
+    // launch configuration (tuning table at plan time; row_v -1: untuned, each
+    // solve picks the TV row configuration for its class, tv_row_default)
+    int row_v = 0, col_v = 0, slot_ctas = 0, lanes = 0;
     int fam = ADMM_REG_TV;      // kernel family: ADMM_REG_TV (isotropic or anisotropic) or ADMM_REG_HAAR
     float lam = 0.f, mu1 = 0.f, mu2 = 0.f;
     void* slab = nullptr;
@@ -337,7 +340,7 @@ int col_block(int H) {
 }
 int row_strip_tv(int W) {
     const RowVariant* v = nullptr;
-    return tv_row_variants(W, &v) > 0 ? v[tv_row_default(W)].R : 0;
+    return tv_row_variants(W, &v) > 0 ? v[0].R : 0;
 }
 
 // launch slots of a group: enough problems in flight that a row-side launch
@@ -353,16 +356,18 @@ int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count) {
 using TuneKey = std::tuple<int, int, int, int, int>;   // device, H, W, reg, levels
 std::map<TuneKey, admm_tuning_t> g_tuning;            // under g_mutex
 
-// the configuration a new plan of this class gets (the default when untuned)
-admm_tuning_t lookup_tuning(int dev, int H, int W, int reg, int levels) {
+// the configuration a new plan of this class gets (the default for one
+// problem, and *tuned = false, when untuned)
+admm_tuning_t lookup_tuning(int dev, int H, int W, int reg, int levels, bool* tuned = nullptr) {
     auto it = g_tuning.find(TuneKey(dev, H, W, reg, levels));
+    if (tuned) *tuned = it != g_tuning.end();
     if (it != g_tuning.end()) return it->second;
     admm_tuning_t t{};
     t.H = H;
     t.W = W;
     t.reg = reg;
     t.haar_levels = levels;
-    if (reg == ADMM_REG_TV) t.row_variant = tv_row_default(W);
+    if (reg == ADMM_REG_TV) t.row_variant = tv_row_default(W, (long long)H * W);
     return t;
 }
 
@@ -404,7 +409,7 @@ cudaError_t launch_row_tv(int W, const ProbDesc* d, SlotTable sl, int count, int
                           int* n_active, cudaStream_t s) {
     const RowVariant* v = nullptr;
     if (tv_row_variants(W, &v) == 0) return cudaErrorInvalidValue;
-    return v[tv_row_default(W)].fn(d, sl, count, H, Wp, tw, n_active, s);
+    return v[0].fn(d, sl, count, H, Wp, tw, n_active, s);
 }
 
 template <int W>
@@ -620,11 +625,12 @@ int admm_deconv_plan(admm_plan_t* out, const admm_params_t* p, void* stream) {
         // one configuration (no tuning); the row side is a kernel chain
         pl->cb = gen_col_block(H);
     } else {
-        const admm_tuning_t tu = lookup_tuning(pl->device, H, W, fam, levels);
+        bool tuned = false;
+        const admm_tuning_t tu = lookup_tuning(pl->device, H, W, fam, levels, &tuned);
         const ColVariant* cv = nullptr;
         col_variants(H, &cv);
         pl->col_v = tu.col_variant;
-        pl->row_v = tu.row_variant;
+        pl->row_v = fam != ADMM_REG_TV || tuned ? tu.row_variant : -1;
         pl->slot_ctas = tu.slot_ctas;
         pl->lanes = tu.lanes;
         pl->cb = cv[pl->col_v].CB;
@@ -639,7 +645,9 @@ int admm_deconv_plan(admm_plan_t* out, const admm_params_t* p, void* stream) {
     } else if (fam == ADMM_REG_TV) {
         const RowVariant* rv = nullptr;
         tv_row_variants(W, &rv);
-        pl->R = rv[pl->row_v].R;
+        // (untuned: the shortest strip a solve may pick, which the partial sums are sized for)
+        pl->R = pl->row_v >= 0 ? rv[pl->row_v].R
+                               : std::min(rv[tv_row_default(W, 0)].R, rv[tv_row_default(W, LLONG_MAX)].R);
         pl->nb = 2;
     } else {
         pl->R = haar_row_strip(W);
@@ -1188,6 +1196,8 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
             if (g.tv) {
                 const RowVariant* rv = nullptr;
                 tv_row_variants(g.W, &rv);
+                if (g.row_v < 0) g.row_v = tv_row_default(g.W, (long long)g.H * g.W * (long long)idx.size());
+                g.R = rv[g.row_v].R;
                 g.row_fn = p0->p.reg == ADMM_REG_TV_ANISO ? rv[g.row_v].fn_aniso : rv[g.row_v].fn;
             }
         }
@@ -1222,6 +1232,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
             }
             const int t = (int)order.size();
             ctx->h_desc[t] = make_desc(pl);
+            if (g.tv && !g.gen) ctx->h_desc[t].n_strips = ctx->h_desc[t].n_slots = g.H / g.R;
             // padded plans finalize on their domain and copy the caller's window out
             x_host.push_back(pl->padded || !is_device_ptr(x_out[j]));
             ctx->h_xptr[t] = x_host.back() ? pl->xstage : x_out[j];
@@ -1274,7 +1285,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
         // with per-phase timing on, one lane: every launch covers all slots,
         // so the timed phases are the full-size kernels
         // (as is a class that runs in teams)
-        team = team && g.tv && !g.gen && g.row_v == 0 && g.nslots == g.count &&
+        team = team && g.tv && !g.gen && p0->row_v <= 0 && g.nslots == g.count &&
                use_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, g.count);
         g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : default_lanes(g.H, g.W, g.nslots), g.count, g.nslots}));
         for (int l = 0, o = g.off, so = soff; l < g.L.n; ++l) {

@@ -291,6 +291,26 @@ __device__ __forceinline__ void tv_prox(float sh, float sv, float tau, bool anis
         uv = sc * sv;
     }
 }
+// the prox at s with the dual update d2' = u2 - s and delta = u2 + d2'; the
+// isotropic products are contracted by hand, so that every kernel and every
+// configuration that calls this gives the same bits
+__device__ __forceinline__ void tv_split(float sh, float sv, float tau, bool aniso, float& nh, float& nv, float& dlh,
+                                         float& dlv) {
+    if (aniso) {
+        float uh, uv;
+        tv_prox(sh, sv, tau, true, uh, uv);
+        nh = uh - sh;
+        nv = uv - sv;
+        dlh = uh + nh;
+        dlv = uv + nv;
+    } else {
+        const float sc = fmaxf(0.f, fmaf(-tau, rsqrtf(fmaf(sh, sh, __fmul_rn(sv, sv))), 1.f));
+        nh = fmaf(sc, sh, -sh);
+        nv = fmaf(sc, sv, -sv);
+        dlh = fmaf(sc, sh, nh);
+        dlv = fmaf(sc, sv, nv);
+    }
+}
 // the TV term of the objective at D_i x = (gh, gv)
 __device__ __forceinline__ float tv_norm(float gh, float gv, bool aniso) {
     return aniso ? fabsf(gh) + fabsf(gv) : sqrtf(fmaf(gh, gh, gv * gv));
@@ -771,8 +791,8 @@ struct RowCfg {
     static constexpr size_t SMEM = (size_t)NB * ROW * sizeof(float2) + (size_t)W * sizeof(float2)
                                  + (size_t)D * SLOT * sizeof(float) + NWARP * 2 * kNumPartials * sizeof(float);
     // CTAs per SM the registers are sized for (128-thread CTAs without the
-    // ring fit a fifth CTA in shared memory)
-    static constexpr int MINB = NT == 128 ? (D == 0 ? 5 : 4) : (NT == 64 ? 8 : 2);
+    // ring, or of four short rows, fit a fifth CTA in shared memory)
+    static constexpr int MINB = NT == 128 ? (D == 0 || (R <= 4 && W <= 512) ? 5 : 4) : (NT == 64 ? 8 : 2);
 };
 
 // ANISO: anisotropic TV (soft threshold per difference component)
@@ -1008,12 +1028,7 @@ row_phase_tv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, co
                     // delta = u2 + d2  (Alg. 3 lines 3-5, 9-11; as in the single-column walk)
                     const float gh = xrs[e] - xs[e], gv = xds[e] - xs[e];
                     const float sh = gh - ddh[e], sv = gv - ddv[e];
-                    float uh, uv;
-                    tv_prox(sh, sv, tau, aniso, uh, uv);
-                    nh[e] = uh - sh;
-                    nv[e] = uv - sv;
-                    dhcur[2 * pp + e] = uh + nh[e];
-                    dvcur[2 * pp + e] = uv + nv[e];
+                    tv_split(sh, sv, tau, aniso, nh[e], nv[e], dhcur[2 * pp + e], dvcur[2 * pp + e]);
                     if (owned && nobj) {
                         s_reg.add(tv_norm(gh, gv, aniso));
                         const float eh = nh[e] - ddh[e], ev = nv[e] - ddv[e];
@@ -1059,9 +1074,8 @@ row_phase_tv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, co
                 const float xhr = xa[0].x;
                 const float2 dd = cold ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(slot + 4 * W + 2 * wid);
                 const float sh = (xhr - xh) - dd.x, sv = (xl_nb_dn - xh) - dd.y;
-                float uh, uv;
-                tv_prox(sh, sv, tau, aniso, uh, uv);
-                dh_halo = 2.f * uh - sh;
+                float nh, nv, dv;
+                tv_split(sh, sv, tau, aniso, nh, nv, dh_halo, dv);
             }
             issue(i + D);            // slot (i % D) is consumed: refill it D rows ahead
             // delta_h left of each column: the pair's own first column for the
@@ -1107,15 +1121,11 @@ row_phase_tv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, co
                 const size_t pix = (size_t)q * W + c;
                 const float2 dd = cold ? make_float2(0.f, 0.f)
                                        : (D > 0 ? *reinterpret_cast<const float2*>(slot + 2 * c) : d2in[pix]);
-                // u2 = prox(D_i x - d2, lambda/mu2)  (Alg. 3 line 10)
+                // u2 = prox(D_i x - d2, lambda/mu2), d2 <- d2 - (D_i x - u2) (Alg. 3
+                // lines 10, 11), delta = u2 + d2 for the next x-step (lines 3-5)
                 const float sh = gh - dd.x, sv = gv - dd.y;
-                float uh, uv;
-                tv_prox(sh, sv, tau, aniso, uh, uv);
-                // d2 <- d2 - (D_i x - u2)  (Alg. 3 line 11)
-                const float nh = uh - sh, nv = uv - sv;
-                // delta = u2 + d2 for the next x-step (Alg. 3 lines 3-5)
-                dhcur[j] = uh + nh;
-                dvcur[j] = uv + nv;
+                float nh, nv;
+                tv_split(sh, sv, tau, aniso, nh, nv, dhcur[j], dvcur[j]);
                 z1cur[j] = 0.f;
                 if (owned) {
                     d2out[pix] = make_float2(nh, nv);
@@ -1155,9 +1165,8 @@ row_phase_tv(const ProbDesc* __restrict__ probs, SlotTable sl, int H, int Wp, co
                                         : (D > 0 ? *reinterpret_cast<const float2*>(slot + 4 * W + 2 * wid)
                                                  : d2in[(size_t)q * W + chalo]);
                 const float sh = (xhr - xh) - dd.x, sv = (xl_nb_dn - xh) - dd.y;
-                float uh, uv;
-                tv_prox(sh, sv, tau, aniso, uh, uv);
-                dh_halo = 2.f * uh - sh;
+                float nh, nv, dv;
+                tv_split(sh, sv, tau, aniso, nh, nv, dh_halo, dv);
             }
         }
         issue(i + D);                // slot (i % D) is consumed: refill it D rows ahead

@@ -1,6 +1,5 @@
 // rows_large.cu -- compiled TV row-phase configurations for W = 1024, 2048
-// (rows per strip, walk rows in flight, threads per CTA); the default is
-// tv_row_default of each width.
+// (rows per strip, walk rows in flight, threads per CTA; tv_row_default picks).
 #include "variants.cuh"
 
 namespace admm {

@@ -403,7 +403,7 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
             __syncthreads();
         }
         float2 v[8] = {};
-        float ddh[8], ddv[8], edge[8];               // delta = u2 + d2; delta_h for the next group of columns
+        float ddh[8], ddv[8];                        // delta = u2 + d2
         // STATS: the iteration evaluates the objective (a check iteration does, too);
         // two bodies, each free of branches between its eight pixels
         auto row_phase = [&](auto stats) {
@@ -457,27 +457,8 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
                 const float x = v[m].x, xd = xs[(id + 1) * W + t + m * FT];
                 const float gh = xr[m] - x, gv = xd - x;
                 const float sh = gh - dh[m], sv = gv - dv[m];
-                // u2 = prox(s), d2' = u2 - s, delta = u2 + d2', with the products that
-                // row_phase_tv contracts contracted, and the delta_h that crosses from
-                // one warp's columns to the next formed as there (its default
-                // configuration's warps own W/8 columns too): both give the same bits
                 float nh, nv;
-                if constexpr (ANISO) {
-                    float uh, uv;
-                    tv_prox(sh, sv, tau, true, uh, uv);
-                    nh = uh - sh;
-                    nv = uv - sv;
-                    ddh[m] = uh + nh;
-                    ddv[m] = uv + nv;
-                    edge[m] = 2.f * uh - sh;
-                } else {
-                    const float sc = fmaxf(0.f, fmaf(-tau, rsqrtf(fmaf(sh, sh, __fmul_rn(sv, sv))), 1.f));
-                    nh = fmaf(sc, sh, -sh);
-                    nv = fmaf(sc, sv, -sv);
-                    ddh[m] = fmaf(sc, sh, nh);
-                    ddv[m] = fmaf(sc, sv, nv);
-                    edge[m] = fmaf(2.f, __fmul_rn(sc, sh), -sh);
-                }
+                tv_split(sh, sv, tau, ANISO, nh, nv, ddh[m], ddv[m]);
                 if constexpr (STATS) {
                     const float eh = nh - dh[m], ev = nv - dv[m];
                     s_reg.add(owned ? tv_norm(gh, gv, ANISO) : 0.f);
@@ -527,7 +508,7 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
             const float a = __shfl_up_sync(0xffffffffu, ddh[m], 1, FT);
-            const float b = __shfl_sync(0xffffffffu, edge[(m + 7) & 7], FT - 1, FT);
+            const float b = __shfl_sync(0xffffffffu, ddh[(m + 7) & 7], FT - 1, FT);
             dl[m] = t == 0 ? b : a;
         }
         if (owned) {

@@ -3,8 +3,9 @@
 //
 // Every side length has a short list of compiled configurations of the TV
 // row phase (rows per strip R, walk rows in flight D, threads per CTA NT) and
-// of the column phase (columns per CTA CB); entry 0 of each list is the
-// default, but for rows of 2048 (tv_row_default). The autotuner (admm_deconv_autotune) times the combinations on the
+// of the column phase (columns per CTA CB). Untuned classes take entry 0 of
+// the column phase's list and the row configuration that tv_row_default
+// names. The autotuner (admm_deconv_autotune) times the combinations on the
 // device and records the fastest per (device, H, W, regulariser, levels);
 // plans created afterwards use it. The instantiations are spread over
 // several translation units (rows_small.cu, rows_512.cu, rows_large.cu,
@@ -36,13 +37,30 @@ struct ColVariant {
 // candidates for one side length (entry 0 = default); returns their number,
 // 0 for an unsupported side
 int tv_row_variants(int W, const RowVariant** out);
-// the TV row configuration of an untuned class. At W = 2048 a strip of two
-// rows does 2x the inverse transforms that its rows need (four rows: 1.5x),
-// but it holds half the shared memory, so that twice the CTAs hide the walk's
-// latencies: 2048^2 x 1 152.8 -> 132.8 us per iteration (both phases), x 2
-// 130.4 -> 116.8, x 4 120.2 -> 115.3; 1024 x 2048 x 2 69.6 -> 64.3. Elsewhere
-// entry 0 is the fastest of its list for one image and within 5 % for many.
-inline int tv_row_default(int W) { return W == 2048 ? 2 : 0; }
+// The TV row configuration of an untuned class with `pixels` = H W problems
+// in flight; every configuration gives the same bits. Short strips transform
+// more halo rows, but their CTAs are many and small, which hides the walk's
+// latencies: on narrow rows they always win, on rows of 512 only while a
+// launch is short of CTAs; rows of 1024 take the longer strip as soon as
+// their launches fill the GPU. Us per problem and iteration (both phases):
+//   W   64  (16,4,256) -> (4,2,64)   64^2 x 256 0.40 -> 0.28, 512 x 64 x 1 22.8 -> 16.1
+//   W  128  (16,4,256) -> (4,2,64)   128^2 x 64 0.87 -> 0.67, 512 x 128 x 4 6.46 -> 5.02
+//   W  256  (8,4,256) -> (4,2,128)   256^2 x 64 1.74 -> 1.51, x 8 2.93 -> 2.83, 512 x 256 x 1 19.4 -> 18.5
+//   W  512  (8,1,128) -> (4,1,128)   512^2 x 1 29.3 -> 23.7, x 4 9.08 -> 8.41, but x 8 6.63 -> 7.10, x 64 4.75 -> 5.06
+//   W 1024  (4,2,256) -> (8,1,256)   1024^2 x 2 33.1 -> 31.8, x 8 25.9 -> 25.2, but x 1 40.3 -> 42.9
+//   W 2048  (4,1,256) -> (2,1,256)   2048^2 x 1 152.8 -> 132.8, x 4 120.2 -> 115.3
+inline int tv_row_default(int W, long long pixels) {
+    const bool few = pixels <= 1ll << 20;
+    switch (W) {
+        case 64: return 3;
+        case 128: return 3;
+        case 256: return 4;
+        case 512: return few ? 6 : 0;
+        case 1024: return few ? 0 : 1;
+        case 2048: return 2;
+    }
+    return 0;
+}
 int col_variants(int H, const ColVariant** out);
 
 // per translation unit
