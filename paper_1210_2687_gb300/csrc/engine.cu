@@ -978,15 +978,16 @@ int admm_deconv_set_state(admm_plan_t plan, const float* state, void* stream) {
 
 // Whether `count` problems of a small TV class run on teams: as many as are
 // resident at once, or twice that with clusters (a second round of teams, which
-// the hardware starts as the first ones end). Beyond it the general kernels,
-// whose iteration costs about the same for one image as for a few dozen, are
-// faster. Per iteration of the whole batch, team / general: 64 x 64: 1 image 3.9
-// / 19.2 us, 32: 5.9 / 25, 64 (two rounds): 12 / 25; 128 x 128: 1: 5.7 / 20, 16
-// (two rounds): 14 / 24, 32 (four): 28 / 28; 256 x 256: 1: 8.5 / 18.4, 4 (two
-// rounds): 17 / 18.7.
+// the hardware starts as the first ones end) where the rows are no more than
+// 128. Beyond it the general kernels, whose iteration costs about the same for
+// one image as for a few dozen, are faster. Per iteration of the whole batch,
+// team / general (us): 64 x 64: 1 image 3.9 / 17, 36: 9.0 / 18.7; 128 x 128: 4:
+// 7.3 / 17.9, 9: 9.1 / 18.8, 18 (two rounds): 16.7 / 20.2; 128 x 256: 9: 16.6 /
+// 19.5, 18: 25.7 / 24.8; 256 x 128: 9: 19.2 / 19.4, 18: 30.2 / 24.5; 256 x 256:
+// 1: 9.3 / 17.1, 2: 9.8 / 17.7.
 static bool use_tv_team(int H, int W, bool aniso, int count) {
     const int cap = tv_team_capacity(H, W, aniso);
-    return count <= cap * (tv_team_cluster(H, W) ? 2 : 1);
+    return count <= cap * (tv_team_cluster(H, W) && H <= 128 ? 2 : 1);
 }
 
 // One size class of a batch: problems [off, off + count) of the descriptor
