@@ -386,7 +386,11 @@ ADMM_API int admm_deconv_get_launch_overlap(void);
  * chooses how many problems of a size class iterate at once, aiming for a
  * number of row-side CTAs per launch. A tuning table, one entry per
  * (device, H, W, regulariser, levels), says which configuration new plans of
- * that class use; untuned classes use index 0 of each list and 2400 CTAs.
+ * that class use; untuned classes use column index 0, 9600 CTAs and the row
+ * configuration that suits the width and the number of problems of the call
+ * (get_tuning reports the one for a single problem). Every configuration gives
+ * the same iterates. Calls of few small TV images (sides up to 256) keep each
+ * image on one team of CTAs and use the table for their layout only.
  * Plans keep the configuration they were created with, and a batch groups
  * plans by shape AND configuration. The table is library-global. Entries are
  * per kernel family: plans of ADMM_REG_TV_ANISO use the ADMM_REG_TV entry,

@@ -1286,7 +1286,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
         // with per-phase timing on, one lane: every launch covers all slots,
         // so the timed phases are the full-size kernels
         // (as is a class that runs in teams)
-        team = team && g.tv && !g.gen && p0->row_v <= 0 && g.nslots == g.count &&
+        team = team && g.tv && !g.gen && g.nslots == g.count &&
                use_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, g.count);
         g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : default_lanes(g.H, g.W, g.nslots), g.count, g.nslots}));
         for (int l = 0, o = g.off, so = soff; l < g.L.n; ++l) {

@@ -128,3 +128,18 @@ def test_padded_and_not_finite(ad):
     a, b = (_run(ad, k, [(psf, y, m), _problem(64, 64, 6)], dict(max_iters=10)) for k in (False, True))
     assert [r.status for r in a[2]] == [r.status for r in b[2]] == [ad.ADMM_ENONFINITE, 0]
     assert (a[0][1] == b[0][1]).all()
+
+
+@pytest.mark.parametrize("H,W", [(64, 64), (128, 256), (256, 256)])
+def test_tuned_classes(ad, H, W):
+    p = [_problem(H, W, 13)]
+    args = dict(max_iters=25, stop="rel_x", tol=0.0, check_every=4)
+    want = _run(ad, True, p, args)
+    prev = ad.admm_deconv_get_tuning(H, W, "tv")
+    keys = ("H", "W", "reg", "haar_levels", "row_variant", "col_variant", "slot_ctas", "lanes")
+    try:
+        for rv, cv in ((1, 0), (2, 1), (0, 3)):
+            ad.admm_deconv_set_tuning({**{k: prev[k] for k in keys}, "row_variant": rv, "col_variant": cv})
+            _same(_run(ad, False, p, args), want)
+    finally:
+        ad.admm_deconv_set_tuning({k: prev[k] for k in keys})
