@@ -335,6 +335,11 @@ ADMM_API int admm_deconv_warm_start(admm_plan_t plan, const float* x0, const flo
                                   second) and each problem retires with
                                   ADMM_ETIMEOUT, the device staying usable; the
                                   option then resets to 0                         */
+#define ADMM_OPT_TEST_CNN_STALL 4 /* the same for the warm-start network: value 1
+                                  makes one CTA of the next pass's second layer
+                                  (widths that strips of 128 columns fit) withhold
+                                  an input row, so that its waits run out (a few
+                                  seconds); the option then resets to 0           */
 
 /*
  * admm_deconv_set_option -- set a library-wide option (see ADMM_OPT_*).

@@ -62,6 +62,7 @@ EXPORTED = ("admm_deconv_plan", "admm_deconv_solve", "admm_deconv_solve_batch",
 ADMM_OPT_MAX_SLOTS = 1
 ADMM_OPT_FAIL_ALLOC = 2
 ADMM_OPT_TEST_STALL = 3
+ADMM_OPT_TEST_CNN_STALL = 4
 
 
 class admm_params_t(ctypes.Structure):

@@ -67,6 +67,7 @@ long long param_offset(int l) {
 long long param_count() { return param_offset(kLayers); }
 
 std::mutex g_cnn_mutex;
+int g_cnn_test_stall = 0;            // ADMM_OPT_TEST_CNN_STALL: armed for the next pass (under g_cnn_mutex)
 long long g_cnn_launches = 0;
 
 int fail(cudaError_t) { return ADMM_ECUDA; }
@@ -152,6 +153,7 @@ constexpr int kWsBatch = 16;
 struct StartOut {
     float s0, s1, s2;
     int separate;
+    int test_stall;              // test hook (ADMM_OPT_TEST_CNN_STALL): CTA 0 withholds an input row
     float* x0;
     float* d0;
     float* px0[kWsBatch];
@@ -673,7 +675,7 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
                     fence_async_shared();
                     __syncwarp();
                 }
-                if (lane == 0) {
+                if (lane == 0 && !(st.test_stall && blockIdx.x == 0 && n == 1)) {
                     const uint32_t bar = sh_addr(&full[s]);
                     if (inside) {
                         const uint32_t bytes = (uint32_t)(hi - lo) * 16u;
@@ -718,9 +720,11 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
         // one input row in the rotation PH of the slots
         auto row = [&](auto rotation, bool first, bool last) -> bool {
             constexpr int PH = decltype(rotation)::value, UP = (PH + 1) % 3, DOWN = (PH + 2) % 3;   // slots of rows r + 1, r - 1
-            if (!mbar_wait_bounded(sh_addr(&full[s]), fp) || !slot_clear(UP) ||
-                (first && !(slot_clear(PH) && slot_clear(DOWN))))
-                return false;
+            const bool go = mbar_wait_bounded(sh_addr(&full[s]), fp) && slot_clear(UP) &&
+                            (!first || (slot_clear(PH) && slot_clear(DOWN)));
+            // one answer for the warp: where the limit passes as the phase completes,
+            // some lanes see it and some do not
+            if (!__all_sync(0xffffffffu, go)) return false;
             tc_fence_after();
             const uint64_t a0 = a_in + s * (C::STAGE / 16);
             const uint64_t b0 = b_in + (PH == 0 ? 1 : (PH == 1 ? 0 : 2)) * COUT;         // window start
@@ -1020,10 +1024,9 @@ conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__
         int i = 0;
         for (int t = blockIdx.x; t < ntiles; t += G, ++i) {
             const int s = i % kWgStages;
-            if (!mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((i / kWgStages) & 1))) {
-                ok = false;
-                break;
-            }
+            // (one answer for the warp, as its lanes meet again below)
+            ok = __all_sync(0xffffffffu, mbar_wait_bounded(sh_addr(&full[s]), (uint32_t)((i / kWgStages) & 1)));
+            if (!ok) break;
             const uint4* g4 = reinterpret_cast<const uint4*>(sm + s * C::STAGE + C::ASTRIDE);
 #pragma unroll 4
             for (int px = j / PG; px < kWgTW * kWgTH; px += 64 / PG) {
@@ -1506,6 +1509,9 @@ int pack_all(admm_cnn_s* n, cudaStream_t s) {
 // predicted start.
 int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, float* out, const StartOut* st, cudaStream_t s) {
     const bf16* cur = n->a0;
+    StartOut stall{};                    // (the test hook serves one pass)
+    stall.test_stall = g_cnn_test_stall;
+    g_cnn_test_stall = 0;
     for (int l = 0; l < kLayers; ++l) {
         const float* b = n->params + param_offset(l) + (long long)layer_cout(l) * layer_cin(l) * 9;
         if (l == kLayers - 1) {
@@ -1519,7 +1525,8 @@ int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, float* out, co
             if (l == 0)
                 CKC((conv_tc<8, kModeReluBf16>(true, cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
             else
-                CKC((conv_rows<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
+                CKC((conv_rows<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s,
+                                                  l == 1 ? stall : StartOut{})));
             cur = dst;
         }
     }
@@ -1815,6 +1822,11 @@ namespace admm {
 // the driver's tensor-map encoder, for the other translation units (null when
 // the driver does not provide it)
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encode_fn() { return tensor_map_encoder(); }
+
+void cnn_test_stall(int value) {
+    std::lock_guard<std::mutex> lk(g_cnn_mutex);
+    g_cnn_test_stall = value;
+}
 
 bool ws_loaded() {
     std::lock_guard<std::mutex> lk(g_ws_mutex);

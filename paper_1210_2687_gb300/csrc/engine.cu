@@ -39,6 +39,7 @@ using namespace admm;
 
 namespace admm {
 // the learned warm start of admm_warmstart_load (cnn.cu)
+void cnn_test_stall(int value);
 bool ws_loaded();
 int ws_batch_limit(int H, int W);
 int ws_predict_starts(int count, int H, int W, const float* const* ybar, const uint8_t* const* mask,
@@ -1533,6 +1534,11 @@ int admm_deconv_set_option(int option, long long value) {
     if (option == ADMM_OPT_TEST_STALL) {
         if (value != 0 && value != 1) return ADMM_EINVAL;
         g_test_stall = (int)value;
+        return ADMM_OK;
+    }
+    if (option == ADMM_OPT_TEST_CNN_STALL) {
+        if (value != 0 && value != 1) return ADMM_EINVAL;
+        cnn_test_stall((int)value);
         return ADMM_OK;
     }
     return ADMM_EINVAL;
