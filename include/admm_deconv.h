@@ -58,7 +58,10 @@ extern "C" {
                                         (the bulk copies of its spectrum rows) and the frame
                                         synthesis tile (its TMA halo boxes) wait at most
                                         about a second; a problem whose wait ran out
-                                        retires with this status (also in res->status)     */
+                                        retires with this status (also in res->status). So
+                                        do the learned start's network (no problem of the
+                                        call is solved then) and the barriers of small TV
+                                        images that share no cluster (256 x 256)           */
 
 /* ---- enums -------------------------------------------------------------- */
 #define ADMM_REG_TV     0   /* isotropic TV, eq. unconstrained_TV_uBC            */

@@ -40,6 +40,17 @@ extern "C" {
 
 typedef struct admm_cnn_s* admm_cnn_t;
 
+/*
+ * Device waits. Every wait of the network's kernels is bounded (about a
+ * second). One that runs out is reported as ADMM_ETIMEOUT by the call itself
+ * where it waits for the device (admm_cnn_gradients, admm_cnn_train_step with
+ * a loss, admm_cnn_get_params) and otherwise by the next call on the network,
+ * which then does nothing else; what the calls since then have written is not
+ * valid, and training steps since then are left out. The state is clear after
+ * the report. admm_deconv_solve_batch with a learned start returns it before
+ * it solves anything, in the status of every result too.
+ */
+
 /* Number of FP32 parameters of the network (57252). */
 ADMM_API long long admm_cnn_param_count(void);
 

@@ -28,6 +28,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -320,6 +321,19 @@ __device__ __forceinline__ void tmem_zero(uint32_t taddr) {
 __device__ __forceinline__ void layer_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void layer_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The network's error state. A kernel whose bounded wait ran out sets `flag`
+// (device) and *host (pinned), which the next call on the network sees without
+// waiting; parameter updates are left out while the flag is set, and counted.
+struct NetErr {
+    int flag, skipped;
+    int* host;
+};
+__device__ __forceinline__ void net_fail(NetErr* e) {
+    atomicExch(&e->flag, 1);
+    *static_cast<volatile int*>(e->host) = 1;
+    __threadfence_system();
+}
+
 constexpr int kTcTW = 8, kTcTH = 16;                 // output tile (M = 128)
 constexpr int kTcHW = kTcTW + 2, kTcHH = kTcTH + 2;  // halo tile
 constexpr int kTcNP = kTcHW * kTcHH;                 // 180 halo pixels
@@ -327,7 +341,7 @@ constexpr int kTcNP = kTcHW * kTcHH;                 // 180 halo pixels
 // tin: TMA view of the input [img][CIN / 8][H][W][8] (see conv_tc); wpk:
 // [9][COUT][CIN]; MODE kModeReluBf16 (bias, ReLU; out bf16 [img][4][H][W][8]),
 // kModeGateBf16 (gate and out bf16 [img][4][H][W][8]) or kModeOutF32 (bias of
-// the 4 outputs; out float [img][H][W][4]); err: set to 1 if a wait ran out (the CTA then stops,
+// the 4 outputs; out float [img][H][W][4]); err: told if a wait ran out (the CTA then stops,
 // after a bounded wait for its own copies and MMAs still in flight).
 //
 // Pipeline of the CTA's i-th tile (halo buffer and accumulator i & 1): thread
@@ -339,7 +353,7 @@ constexpr int kTcNP = kTcHW * kTcHH;                 // 180 halo pixels
 template <int CIN, int MODE>
 __global__ void __launch_bounds__(128)
 conv3x3_tc(const __grid_constant__ CUtensorMap tin, const bf16* __restrict__ wpk, const float* __restrict__ bias,
-           void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, int* __restrict__ err) {
+           void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, NetErr* __restrict__ err) {
     constexpr int COUT = MODE == kModeOutF32 ? 16 : 32, CH = CIN / 8;
     constexpr int BOXBYTES = CH * kTcNP * 16;                  // one halo box
     constexpr int ABYTES = (BOXBYTES + 127) / 128 * 128;        // (each halo buffer on a 128-byte boundary)
@@ -516,7 +530,7 @@ conv3x3_tc(const __grid_constant__ CUtensorMap tin, const bf16* __restrict__ wpk
         __syncthreads();             // accumulator b is free for tile + 2 G's MMAs
     }
     if (!ok && tid == 0) {
-        atomicExch(err, 1);
+        net_fail(err);
         // let this CTA's own copies and MMAs still in flight finish (bounded)
         // before its tensor memory is released
         for (int b = 0; b < 2; ++b) {
@@ -577,7 +591,7 @@ struct RowsCfg {
 template <int CIN, int MODE>
 __global__ void __launch_bounds__(192, 3)
 conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const float* __restrict__ bias,
-             void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, int* __restrict__ err,
+             void* __restrict__ out, const bf16* __restrict__ gate, int H, int W, int count, NetErr* __restrict__ err,
              const __grid_constant__ StartOut st) {
     using C = RowsCfg<CIN, MODE>;
     constexpr int COUT = C::COUT, PL = C::PL, S = kRowStages;
@@ -849,7 +863,7 @@ conv3x3_rows(const bf16* __restrict__ in, const bf16* __restrict__ wpk, const fl
     ok = __syncthreads_and(mbar_wait_bounded(sh_addr(&done), 0u) && ok) != 0;
     if (!ok && tid == 0) {
         // a wait ran out: let the copies still in flight land (bounded) before leaving
-        atomicExch(err, 1);
+        net_fail(err);
         for (int k = max(used, asked - S); k < asked; ++k)
             mbar_wait_bounded(sh_addr(&full[k % S]), (uint32_t)((k / S) & 1));
     }
@@ -923,7 +937,7 @@ __host__ __device__ constexpr int wgrad_part(int cin, int cout) { return 9 * cin
 template <bool GA, int PA, int PG>
 __global__ void __launch_bounds__(128)
 conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tg,
-                 float* __restrict__ part, int cin, int cout, int H, int W, int images, int* __restrict__ err) {
+                 float* __restrict__ part, int cin, int cout, int H, int W, int images, NetErr* __restrict__ err) {
     using C = WgradCfg<GA, PA, PG>;
     extern __shared__ unsigned char wg_raw[];
     __shared__ __align__(8) unsigned long long full[kWgStages], empty[kWgStages], done;
@@ -1051,7 +1065,7 @@ conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__
     if (!ok) {
         // a wait ran out: let the copies still in flight land (bounded) before leaving
         if (tid == 0) {
-            atomicExch(err, 1);
+            net_fail(err);
             for (int i = asked > kWgStages ? asked - kWgStages : 0; i < asked; ++i)
                 mbar_wait_bounded(sh_addr(&full[i % kWgStages]), (uint32_t)((i / kWgStages) & 1));
         }
@@ -1221,9 +1235,13 @@ cnn_loss_kernel(const float* __restrict__ o, const float* __restrict__ tg, float
 // ---------------------------------------------------------------------------
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ gd, float* __restrict__ m,
                             float* __restrict__ v, long long n, float lr, float b1, float b2, float eps,
-                            float c1, float c2) {
+                            float c1, float c2, NetErr* __restrict__ err) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    if (err->flag) {                     // the gradients are not whole: no step
+        if (i == 0) ++err->skipped;
+        return;
+    }
     const float gi = gd[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
     const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -1345,7 +1363,7 @@ cudaError_t launch_layer(void (*kern)(KArgs...), bool first, int grid, int block
 // [plane][halo row][halo column][8 channels].
 template <int CIN, int MODE>
 cudaError_t conv_tc(bool first, const bf16* in, const bf16* w, const float* bias, void* out, const bf16* gate,
-                    int count, int H, int W, int sms, int* err, cudaStream_t s) {
+                    int count, int H, int W, int sms, NetErr* err, cudaStream_t s) {
     static int per_sm = 0;
     if (per_sm == 0) {
         // CTAs one SM holds, from the kernel's registers and static shared
@@ -1394,7 +1412,7 @@ bool rows_fit(int W) { return ((W + kStrip - 1) / kStrip) * kStrip * 4 <= W * 5;
 // columns fit the width, else the 8 x 16 tiles of conv3x3_tc
 template <int CIN, int MODE>
 cudaError_t conv_rows(const bf16* in, const bf16* w, const float* bias, void* out, const bf16* gate, int count,
-                      int H, int W, int sms, int* err, cudaStream_t s, const StartOut& st = StartOut{}) {
+                      int H, int W, int sms, NetErr* err, cudaStream_t s, const StartOut& st = StartOut{}) {
     using C = RowsCfg<CIN, MODE>;
     const int strips = (W + kStrip - 1) / kStrip;
     if constexpr (MODE != kModeStart) {
@@ -1418,7 +1436,7 @@ cudaError_t conv_rows(const bf16* in, const bf16* w, const float* bias, void* ou
 // row, planes, H, images), so that a tile lands as [row][plane][column][8].
 template <bool GA, int PA, int PG>
 cudaError_t wgrad(bool first, const bf16* a, const bf16* g, float* part, int cin, int cout, int count, int H, int W,
-                  int grid, int* err, cudaStream_t s) {
+                  int grid, NetErr* err, cudaStream_t s) {
     using C = WgradCfg<GA, PA, PG>;
     cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc<GA, PA, PG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)C::SMEM);
@@ -1464,7 +1482,8 @@ struct admm_cnn_s {
     float* wpart = nullptr;        // weight-gradient partial vectors, one per CTA and layer
     double* loss = nullptr;        // device accumulator
     double* h_loss = nullptr;      // pinned
-    int* tc_err = nullptr;         // set by a tensor-core convolution whose bounded wait ran out
+    NetErr* err = nullptr;         // set by a convolution whose bounded wait ran out
+    int* h_err = nullptr;          // ... and its pinned flag
     std::vector<void*> allocs;
 };
 
@@ -1487,6 +1506,22 @@ int check_shape(const admm_cnn_s* n, int count, int H, int W) {
     if (count <= 0 || H < kTile || W < kTile || H % kTile || W % kTile) return ADMM_EINVAL;
     if ((long long)count * H * W > n->max_px) return ADMM_EINVAL;
     return ADMM_OK;
+}
+
+// a kernel of an earlier call, or of this one once it has been waited for, ran
+// into its limit
+bool net_failed(const admm_cnn_s* n) { return *static_cast<volatile const int*>(n->h_err) != 0; }
+// the code for it, once: waits for the device, takes the steps that were left
+// out off Adam's count and clears the state
+int net_report(admm_cnn_s* n) {
+    NetErr e{};
+    CKC(cudaDeviceSynchronize());
+    CKC(cudaMemcpy(&e, n->err, sizeof(e), cudaMemcpyDeviceToHost));
+    n->adam_t -= e.skipped;
+    CKC(cudaMemset(n->err, 0, offsetof(NetErr, host)));
+    CKC(cudaDeviceSynchronize());
+    *static_cast<volatile int*>(n->h_err) = 0;
+    return ADMM_ETIMEOUT;
 }
 
 int pack_all(admm_cnn_s* n, cudaStream_t s) {
@@ -1516,16 +1551,16 @@ int run_layers(admm_cnn_s* n, int count, int H, int W, bool keep, float* out, co
         const float* b = n->params + param_offset(l) + (long long)layer_cout(l) * layer_cin(l) * 9;
         if (l == kLayers - 1) {
             if (st)
-                CKC((conv_rows<32, kModeStart>(cur, n->wf[l], b, nullptr, nullptr, count, H, W, n->sms, n->tc_err, s,
+                CKC((conv_rows<32, kModeStart>(cur, n->wf[l], b, nullptr, nullptr, count, H, W, n->sms, n->err, s,
                                                *st)));
             else
-                CKC((conv_rows<32, kModeOutF32>(cur, n->wf[l], b, out, nullptr, count, H, W, n->sms, n->tc_err, s)));
+                CKC((conv_rows<32, kModeOutF32>(cur, n->wf[l], b, out, nullptr, count, H, W, n->sms, n->err, s)));
         } else {
             bf16* dst = keep ? n->act[l] : n->act[l & 1];
             if (l == 0)
-                CKC((conv_tc<8, kModeReluBf16>(true, cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s)));
+                CKC((conv_tc<8, kModeReluBf16>(true, cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->err, s)));
             else
-                CKC((conv_rows<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->tc_err, s,
+                CKC((conv_rows<32, kModeReluBf16>(cur, n->wf[l], b, dst, nullptr, count, H, W, n->sms, n->err, s,
                                                   l == 1 ? stall : StartOut{})));
             cur = dst;
         }
@@ -1573,17 +1608,17 @@ int backward(admm_cnn_s* n, int count, int H, int W, const float* target, const 
         float* pt = n->wpart + ra.base[l] * ncta;
         const bf16* a_in = l == 0 ? n->a0 : n->act[l - 1];
         if (l == kLayers - 1)
-            CKC((wgrad<false, 4, 1>(true, a_in, g, pt, kWidth, kOut, count, H, W, ncta, n->tc_err, s)));
+            CKC((wgrad<false, 4, 1>(true, a_in, g, pt, kWidth, kOut, count, H, W, ncta, n->err, s)));
         else if (l == 0)
-            CKC((wgrad<true, 1, 4>(false, a_in, g, pt, kIn, kWidth, count, H, W, ncta, n->tc_err, s)));
+            CKC((wgrad<true, 1, 4>(false, a_in, g, pt, kIn, kWidth, count, H, W, ncta, n->err, s)));
         else
-            CKC((wgrad<false, 4, 4>(false, a_in, g, pt, kWidth, kWidth, count, H, W, ncta, n->tc_err, s)));
+            CKC((wgrad<false, 4, 4>(false, a_in, g, pt, kWidth, kWidth, count, H, W, ncta, n->err, s)));
         if (l == 0) break;
         bf16* gnext = n->gbuf[l & 1];
         if (l == kLayers - 1)
-            CKC((conv_rows<16, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
+            CKC((conv_rows<16, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->err, s)));
         else
-            CKC((conv_rows<32, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->tc_err, s)));
+            CKC((conv_rows<32, kModeGateBf16>(g, n->wb[l], nullptr, gnext, a_in, count, H, W, n->sms, n->err, s)));
         g = gnext;
     }
     wgrad_reduce_kernel<<<blocks, 256, 0, s>>>(n->wpart, n->grads, ncta, ra);
@@ -1607,6 +1642,7 @@ void admm_cnn_destroy(admm_cnn_t net) {
     if (!net) return;
     for (void* p : net->allocs) cudaFree(p);
     if (net->h_loss) cudaFreeHost(net->h_loss);
+    if (net->h_err) cudaFreeHost(net->h_err);
     delete net;
 }
 
@@ -1628,7 +1664,7 @@ int admm_cnn_create(admm_cnn_t* out, long long max_pixels, int training) {
     const long long P = param_count();
     const size_t px = (size_t)max_pixels;
     if ((rc = dalloc(n, &n->params, P)) || (rc = dalloc(n, &n->a0, px * 8)) || (rc = dalloc(n, &n->out, px * 4)) ||
-        (rc = dalloc(n, &n->tc_err, 1)))
+        (rc = dalloc(n, &n->err, 1)))
         return bail(rc);
     for (int l = 0; l < kLayers; ++l) {
         if ((rc = dalloc(n, &n->wf[l], (size_t)9 * layer_coutp(l) * layer_cinp(l)))) return bail(rc);
@@ -1649,7 +1685,16 @@ int admm_cnn_create(admm_cnn_t* out, long long max_pixels, int training) {
         }
     }
     if (cudaMemset(n->params, 0, P * sizeof(float)) != cudaSuccess) return bail(ADMM_ECUDA);
-    if (cudaMemset(n->tc_err, 0, sizeof(int)) != cudaSuccess) return bail(ADMM_ECUDA);
+    if (admm::alloc_fault_fire() || cudaHostAlloc(&n->h_err, sizeof(int), cudaHostAllocMapped) != cudaSuccess) {
+        n->h_err = nullptr;
+        cudaGetLastError();
+        return bail(ADMM_ENOMEM);
+    }
+    *n->h_err = 0;
+    NetErr e{};
+    if (cudaHostGetDevicePointer(&e.host, n->h_err, 0) != cudaSuccess ||
+        cudaMemcpy(n->err, &e, sizeof(e), cudaMemcpyHostToDevice) != cudaSuccess)
+        return bail(ADMM_ECUDA);
     if (pack_all(n, nullptr) != ADMM_OK || cudaDeviceSynchronize() != cudaSuccess) return bail(ADMM_ECUDA);
     *out = n;
     return ADMM_OK;
@@ -1658,6 +1703,7 @@ int admm_cnn_create(admm_cnn_t* out, long long max_pixels, int training) {
 int admm_cnn_set_params(admm_cnn_t net, const float* params) {
     if (!net || !params) return ADMM_EINVAL;
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
+    if (net_failed(net)) return net_report(net);
     const long long P = param_count();
     CKC(cudaMemcpy(net->params, params, P * sizeof(float), cudaMemcpyDefault));
     if (net->training) {
@@ -1675,7 +1721,7 @@ int admm_cnn_get_params(admm_cnn_t net, float* params) {
     if (!net || !params) return ADMM_EINVAL;
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
     CKC(cudaMemcpy(params, net->params, param_count() * sizeof(float), cudaMemcpyDefault));
-    return ADMM_OK;
+    return net_failed(net) ? net_report(net) : ADMM_OK;
 }
 
 int admm_cnn_forward(admm_cnn_t net, int count, int H, int W, const float* ybar, const uint8_t* mask, float* out,
@@ -1684,6 +1730,7 @@ int admm_cnn_forward(admm_cnn_t net, int count, int H, int W, const float* ybar,
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
+    if (net_failed(net)) return net_report(net);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // (the last layer stores 16 bytes per pixel: straight to `out` where that is aligned)
     const bool direct = (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
@@ -1699,12 +1746,14 @@ int admm_cnn_gradients(admm_cnn_t net, int count, int H, int W, const float* yba
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
+    if (net_failed(net)) return net_report(net);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((rc = forward(net, count, H, W, ybar, mask, true, net->out, nullptr, s)) != ADMM_OK) return rc;
     if ((rc = backward(net, count, H, W, target, chan_w, s)) != ADMM_OK) return rc;
     CKC(cudaMemcpyAsync(grads, net->grads, param_count() * sizeof(float), cudaMemcpyDefault, s));
     CKC(cudaMemcpyAsync(net->h_loss, net->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
     CKC(cudaStreamSynchronize(s));
+    if (net_failed(net)) return net_report(net);
     if (loss) *loss = *net->h_loss;
     return ADMM_OK;
 }
@@ -1715,6 +1764,7 @@ int admm_cnn_train_step(admm_cnn_t net, int count, int H, int W, const float* yb
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
+    if (net_failed(net)) return net_report(net);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if ((rc = forward(net, count, H, W, ybar, mask, true, net->out, nullptr, s)) != ADMM_OK) return rc;
     if ((rc = backward(net, count, H, W, target, chan_w, s)) != ADMM_OK) return rc;
@@ -1724,13 +1774,14 @@ int admm_cnn_train_step(admm_cnn_t net, int count, int H, int W, const float* yb
     const float c2 = (float)(1.0 - std::pow(0.999, (double)net->adam_t));
     const long long P = param_count();
     adam_kernel<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(net->params, net->grads, net->m, net->v, P, lr, b1, b2,
-                                                            1e-8f, c1, c2);
+                                                            1e-8f, c1, c2, net->err);
     ++g_cnn_launches;
     CKC(cudaGetLastError());
     if ((rc = pack_all(net, s)) != ADMM_OK) return rc;
     if (loss) {
         CKC(cudaMemcpyAsync(net->h_loss, net->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
         CKC(cudaStreamSynchronize(s));
+        if (net_failed(net)) return net_report(net);
         *loss = *net->h_loss;
     }
     return ADMM_OK;
@@ -1742,6 +1793,7 @@ int admm_cnn_predict_start(admm_cnn_t net, int count, int H, int W, const float*
     std::lock_guard<std::mutex> lk(g_cnn_mutex);
     int rc = check_shape(net, count, H, W);
     if (rc != ADMM_OK) return rc;
+    if (net_failed(net)) return net_report(net);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     StartOut st{};
     st.s0 = scales[0];
@@ -1833,6 +1885,15 @@ bool ws_loaded() {
     return g_ws.loaded;
 }
 
+// whether a pass of the network since the last call of this function ran into
+// the limit of a bounded wait (its stream has been waited for): ADMM_ETIMEOUT,
+// and the state is clear again
+int ws_take_error() {
+    std::lock_guard<std::mutex> lk(g_ws_mutex);
+    std::lock_guard<std::mutex> lk2(g_cnn_mutex);
+    return g_ws.net && net_failed(g_ws.net) ? net_report(g_ws.net) : ADMM_OK;
+}
+
 // images of H x W that one ws_predict_starts call takes: up to 16, and no
 // more than 16 x 512 x 512 pixels (the network's buffers hold about 180 B per
 // pixel)
@@ -1855,8 +1916,14 @@ int ws_predict_starts(int count, int H, int W, const float* const* ybar, const u
     if (cudaGetDevice(&dev) != cudaSuccess) return ADMM_ECUDA;
     const long long hw = (long long)H * W, px = hw * count;
     if (!g_ws.net || g_ws.device != dev || g_ws.cap < px) {
-        if (g_ws.net) admm_cnn_destroy(g_ws.net);
-        g_ws.net = nullptr;
+        if (g_ws.net) {
+            // (its passes of this call are not waited for yet)
+            CKC(cudaDeviceSynchronize());
+            const bool failed = net_failed(g_ws.net);
+            admm_cnn_destroy(g_ws.net);
+            g_ws.net = nullptr;
+            if (failed) return ADMM_ETIMEOUT;
+        }
         const long long cap = std::max(px, 512LL * 512LL);
         admm_cnn_t n = nullptr;
         int rc = admm_cnn_create(&n, cap, 0);

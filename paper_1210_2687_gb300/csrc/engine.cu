@@ -41,6 +41,7 @@ namespace admm {
 // the learned warm start of admm_warmstart_load (cnn.cu)
 void cnn_test_stall(int value);
 bool ws_loaded();
+int ws_take_error();
 int ws_batch_limit(int H, int W);
 int ws_predict_starts(int count, int H, int W, const float* const* ybar, const uint8_t* const* mask,
                       float* const* x0, float* const* d0, cudaStream_t s);
@@ -1150,6 +1151,20 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
     // staging table are prepared by the next flush (before a learned start
     // reads its problem's prepared input, and after the last problem)
     int prep_done = 0, prep_n = 0, prep_maxn = 0;
+    // a learned start that failed fails the call before anything is solved: its
+    // problems start cold again next time, and every result says so
+    std::vector<admm_plan_s*> ws_all;
+    auto learned_failed = [&](int r) -> int {
+        for (admm_plan_s* pl : ws_all) pl->warm_mode = 0;
+        if (res && r == ADMM_ETIMEOUT)
+            for (const std::vector<int>& idx : classes)
+                for (int j : idx) {
+                    res[j] = admm_result_t{};
+                    res[j].status = r;
+                    res[j].objective = NAN;
+                }
+        return r;
+    };
     auto flush_prep = [&]() -> int {
         const int cnt = prep_n - prep_done;
         if (cnt <= 0) return ADMM_OK;
@@ -1231,6 +1246,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
                 if (pl->d2 != pl->d1 + n) return ADMM_ECUDA;
                 pl->warm_mode = 1;
                 ws_pend.push_back(pl);
+                ws_all.push_back(pl);
             }
             const int t = (int)order.size();
             ctx->h_desc[t] = make_desc(pl);
@@ -1278,10 +1294,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
                 return ADMM_OK;
             };
             const int r = learned();
-            if (r != ADMM_OK) {
-                for (admm_plan_s* pl : ws_pend) pl->warm_mode = 0;
-                return r;
-            }
+            if (r != ADMM_OK) return learned_failed(r);
         }
         g.nslots = choose_slots(g.H, g.W, g.tv, g.R, g.slot_ctas, g.count);
         // with per-phase timing on, one lane: every launch covers all slots,
@@ -1325,6 +1338,10 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
     }
     // the host-side tables are reused by the next call
     CK(cudaStreamSynchronize(s));
+    if (!ws_all.empty()) {
+        const int r = ws_take_error();
+        if (r != ADMM_OK) return learned_failed(r);
+    }
 
     // with more problems than slots, problems start as slots free up: the
     // iterations needed by a class are bounded by the sum of its per-slot work
