@@ -337,7 +337,10 @@ ADMM_API int admm_deconv_warm_start(admm_plan_t plan, const float* x0, const flo
                                   CTA, so that the wait for it runs out (about a
                                   second) and each problem retires with
                                   ADMM_ETIMEOUT, the device staying usable; the
-                                  option then resets to 0                         */
+                                  option then resets to 0. A 256 x 256 TV image on
+                                  a team of CTAs: one CTA gives up at the end of
+                                  the first iteration, the others' waits for it
+                                  run out in the second                           */
 #define ADMM_OPT_TEST_CNN_STALL 4 /* the same for the warm-start network: value 1
                                   makes one CTA of the next pass's second layer
                                   (widths that strips of 128 columns fit) withhold

@@ -1142,11 +1142,13 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
     int soff = 0, qbase = 0;
     // A call of one class of small TV images runs each image on a team of CTAs,
     // many iterations per launch (team.cuh): not with per-phase timing, whose
-    // phases are the general kernels', nor with the stall hook, which withholds
-    // one of their copies; and only in the row configuration whose bits the team
-    // kernel reproduces, so that a problem's result does not depend on how many
-    // are solved with it.
-    bool team = classes.size() == 1 && !prof && !t_general && g_test_stall == 0;
+    // phases are the general kernels', and with the stall hook only the teams that
+    // have a bounded barrier (a cluster's is the hardware's). The iterates are those
+    // of the general kernels in any configuration, bit for bit; the objective and the
+    // relative changes are sums in another order, so a stop exactly at the tolerance
+    // may differ with the number of problems of the call (as it may between the
+    // strips of tv_row_default).
+    bool team = classes.size() == 1 && !prof && !t_general;
     // input preparation, batched: items [prep_done, prep_n) of the pinned
     // staging table are prepared by the next flush (before a learned start
     // reads its problem's prepared input, and after the last problem)
@@ -1300,7 +1302,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
         // with per-phase timing on, one lane: every launch covers all slots,
         // so the timed phases are the full-size kernels
         // (as is a class that runs in teams)
-        team = team && g.tv && !g.gen && g.nslots == g.count &&
+        team = team && g.tv && !g.gen && g.nslots == g.count && !(g_test_stall && tv_team_cluster(g.H, g.W)) &&
                use_tv_team(g.H, g.W, g.reg == ADMM_REG_TV_ANISO, g.count);
         g.L.n = prof || team ? 1 : std::max(1, std::min({g.lanes > 0 ? g.lanes : default_lanes(g.H, g.W, g.nslots), g.count, g.nslots}));
         for (int l = 0, o = g.off, so = soff; l < g.L.n; ++l) {

@@ -117,6 +117,14 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
     const ProbDesc& P = probs[pi];
     ProbCtl* const ctl = P.ctl;
     if (ctl->active == 0) return;
+    if (ctl->status == kStatusTimeout) {             // (a wait of another CTA ran out at the end of the last launch)
+        if (rank == 0 && threadIdx.x == 0) {
+            ctl->active = 0;
+            ctl->t_done = device_clock_ns();
+            atomicSub(n_active, 1);
+        }
+        return;
+    }
     extern __shared__ __align__(16) unsigned char cl_raw[];
     float4* tile = reinterpret_cast<float4*>(cl_raw);                      // [H][NC]
     float4* spec = reinterpret_cast<float4*>(cl_raw + C::TILE);            // [GR][Wc]
@@ -195,6 +203,8 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
     // solve; false if a wait ran out (about a second).
     unsigned target = ctl->team_base;
     bool first_bar = true;
+    // (test hook: the last CTA's wait at the launch's second barrier counts as one that ran out)
+    const bool gives_up = !DSM && P.test_stall && rank == C::C - 1;
     auto barrier = [&]() -> bool {
         if constexpr (DSM) {
             cluster_barrier();
@@ -209,7 +219,7 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
                 // other work to leave its SMs. The clock is read every 256 polls.
                 unsigned long long t0 = 0;
                 const unsigned long long limit = first_bar ? 10000000000ull : 1000000000ull;
-                int good = 1;
+                int good = gives_up && !first_bar ? 0 : 1;
                 for (unsigned n = 1;; ++n) {
                     unsigned v;
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->team_bar) : "memory");
@@ -572,7 +582,8 @@ tv_team(const ProbDesc* __restrict__ probs, SlotTable sl, int Wp, const float2* 
     if (rank == 0 && service && lane == 0) {
         ctl->team_base = target;
         ctl->iter = k;
-        if (alive) ctl->status = status;
+        // (0 to this decision's: a wait that ran out in another CTA, at the last barrier alone too, stays)
+        if (status != 0) atomicCAS(&ctl->status, 0, status);
         ctl->have_obj = have_obj;
         ctl->obj = obj;
         ctl->obj_prev = obj_prev;
