@@ -1180,45 +1180,54 @@ wgrad_reduce_kernel(const float* __restrict__ ws, float* __restrict__ grads, int
 // ---------------------------------------------------------------------------
 // loss and its gradient in the output: g = 2 c_k (o - t) / npx (one plane of
 // eight channels, 4 used; its readers take the second plane of a 16-channel
-// operand as zeros outside the tensor map). Bound by its 48 B per pixel. The
-// squared errors are summed per thread as FP32 pairs without rounding error
-// (product and sum split exactly, which keeps about 48 bits: FP64 units are
-// scarce here), per block in FP64, one atomic per block; the grid is a few
-// blocks per SM, not one block per 256 pixels: 4096 atomics on one address and
-// eight FP64 operations per pixel made it 50 us at 16 x 256^2.
+// operand as zeros outside the tensor map). 48 B per pixel and four FMAs on the
+// few FP64 units, where a squared error is exact (48 bits, any finite float's
+// square in range) and so are infinities and NaN. Normal floats are widened with
+// integer instructions, since conversions run on those units as well. One atomic
+// per block; the grid is a few blocks per SM, not one block per 256 pixels: 4096
+// atomics on one address and eight FP64 operations per pixel made it 50 us at
+// 16 x 256^2, now 18 us (26 with conversions).
 // ---------------------------------------------------------------------------
-struct PairSum {
-    float h = 0.f, l = 0.f;
-    // add v * v
-    __device__ __forceinline__ void add_sq(float v) {
-        const float p = v * v, e = fmaf(v, v, -p);
-        const float t = h + p, z = t - h;
-        l += ((h - (t - z)) + (p - z)) + e;
-        h = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-};
+__device__ __forceinline__ bool is_normal(float v) {
+    return (__float_as_uint(v) & 0x7FFFFFFFu) - 0x00800000u < 0x7F000000u;
+}
+// |v| of a normal float: the exponent moved by 1023 - 127, the fraction by 29 bits
+__device__ __forceinline__ double widen_abs(float v) {
+    const uint32_t u = __float_as_uint(v) & 0x7FFFFFFFu;
+    return __hiloint2double((int)((u >> 3) + 0x38000000u), (int)(u << 29));
+}
 
 __global__ void __launch_bounds__(256)
 cnn_loss_kernel(const float* __restrict__ o, const float* __restrict__ tg, float4 cw, bf16* __restrict__ gout,
                 double* __restrict__ loss, long long npx) {
     __shared__ double red[8];
-    PairSum sx, sy, sz, sw;
+    double sx = 0.0, sy = 0.0, sz = 0.0, sw = 0.0;   // sums of the squared errors
     const float s = 2.0f / (float)npx;
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < npx; i += (long long)gridDim.x * 256) {
         const float4 ov = reinterpret_cast<const float4*>(o)[i];
         const float4 tv = __ldcs(reinterpret_cast<const float4*>(tg) + i);
         const float e0 = ov.x - tv.x, e1 = ov.y - tv.y, e2 = ov.z - tv.z, e3 = ov.w - tv.w;
-        sx.add_sq(e0);
-        sy.add_sq(e1);
-        sz.add_sq(e2);
-        sw.add_sq(e3);
+        double d0, d1, d2, d3;
+        if (is_normal(e0) && is_normal(e1) && is_normal(e2) && is_normal(e3)) {
+            d0 = widen_abs(e0);
+            d1 = widen_abs(e1);
+            d2 = widen_abs(e2);
+            d3 = widen_abs(e3);
+        } else {
+            d0 = e0;
+            d1 = e1;
+            d2 = e2;
+            d3 = e3;
+        }
+        sx = fma(d0, d0, sx);
+        sy = fma(d1, d1, sy);
+        sz = fma(d2, d2, sz);
+        sw = fma(d3, d3, sw);
         reinterpret_cast<uint4*>(gout)[i] =
             make_uint4(pack2(__float2bfloat16(s * cw.x * e0), __float2bfloat16(s * cw.y * e1)),
                        pack2(__float2bfloat16(s * cw.z * e2), __float2bfloat16(s * cw.w * e3)), 0u, 0u);
     }
-    double l = (double)cw.x * sx.value() + (double)cw.y * sy.value() + (double)cw.z * sz.value() +
-               (double)cw.w * sw.value();
+    double l = (double)cw.x * sx + (double)cw.y * sy + (double)cw.z * sz + (double)cw.w * sw;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) l += __shfl_down_sync(0xffffffffu, l, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
