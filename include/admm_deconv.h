@@ -397,11 +397,14 @@ ADMM_API int admm_deconv_get_launch_overlap(void);
  * chooses how many problems of a size class iterate at once, aiming for a
  * number of row-side CTAs per launch. A tuning table, one entry per
  * (device, H, W, regulariser, levels), says which configuration new plans of
- * that class use; untuned classes use column index 0, 9600 CTAs and the row
- * configuration that suits the width and the number of problems of the call
- * (get_tuning reports the one for a single problem). Every configuration gives
- * the same iterates. Calls of few small TV images (sides up to 256) keep each
- * image on one team of CTAs and use the table for their layout only.
+ * that class use. An entry with row_variant, col_variant, slot_ctas and lanes
+ * all 0 is the untuned class, as if it were not there: column index 0, 9600
+ * CTAs and the row configuration that suits the width and the number of problems
+ * of the call (rows_per_strip and the like describe a large batch's). Any other
+ * entry fixes its row configuration, whatever the number of problems. Every
+ * configuration gives the same iterates. Calls of few small TV images (sides up
+ * to 256) keep each image on one team of CTAs and use the table for their layout
+ * only.
  * Plans keep the configuration they were created with, and a batch groups
  * plans by shape AND configuration. The table is library-global. Entries are
  * per kernel family: plans of ADMM_REG_TV_ANISO use the ADMM_REG_TV entry,
@@ -411,7 +414,8 @@ typedef struct {
     int    H, W;            /* [in] the size class ...                                        */
     int    reg;             /* [in] ... ADMM_REG_TV or ADMM_REG_HAAR ...                      */
     int    haar_levels;     /* [in] ... and levels (1..4 for Haar, 0 = 4; ignored for TV)     */
-    int    row_variant;     /* index of the TV row-phase configuration of W (0 for Haar)     */
+    int    row_variant;     /* index of the TV row-phase configuration of W (0 for Haar; 0 with
+                               the three fields below 0: chosen by each call)                 */
     int    col_variant;     /* index of the column-phase configuration of H                  */
     int    slot_ctas;       /* row-side CTAs per launch aimed for (0 = default 9600)         */
     int    lanes;           /* independent lanes (graph branches) the class's problems and

@@ -358,23 +358,28 @@ int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count) {
 using TuneKey = std::tuple<int, int, int, int, int>;   // device, H, W, reg, levels
 std::map<TuneKey, admm_tuning_t> g_tuning;            // under g_mutex
 
-// the configuration a new plan of this class gets (the default for one
-// problem, and *tuned = false, when untuned)
+// An entry with every choice 0 is the untuned class: it leaves the rows to each
+// call (tv_row_default), whether it was never set, read back and set again, or
+// the autotuner's winner.
+bool is_untuned(const admm_tuning_t& t) {
+    return t.row_variant == 0 && t.col_variant == 0 && t.slot_ctas == 0 && t.lanes == 0;
+}
+
+// the configuration a new plan of this class gets (*tuned = false: the untuned one)
 admm_tuning_t lookup_tuning(int dev, int H, int W, int reg, int levels, bool* tuned = nullptr) {
     auto it = g_tuning.find(TuneKey(dev, H, W, reg, levels));
-    if (tuned) *tuned = it != g_tuning.end();
+    if (tuned) *tuned = it != g_tuning.end() && !is_untuned(it->second);
     if (it != g_tuning.end()) return it->second;
     admm_tuning_t t{};
     t.H = H;
     t.W = W;
     t.reg = reg;
     t.haar_levels = levels;
-    if (reg == ADMM_REG_TV) t.row_variant = tv_row_default(W, (long long)H * W);
     return t;
 }
 
-// fill the descriptive fields of `t` from its indices; false if an index is
-// out of range for the class
+// fill the descriptive fields of `t` from its indices (an untuned class: the
+// rows of a large batch); false if an index is out of range for the class
 bool describe_tuning(admm_tuning_t* t) {
     const ColVariant* cv = nullptr;
     const int nc = col_variants(t->H, &cv);
@@ -386,9 +391,10 @@ bool describe_tuning(admm_tuning_t* t) {
         const RowVariant* rv = nullptr;
         const int nr = tv_row_variants(t->W, &rv);
         if (t->row_variant < 0 || t->row_variant >= nr) return false;
-        t->rows_per_strip = rv[t->row_variant].R;
-        t->walk_depth = rv[t->row_variant].D;
-        t->row_threads = rv[t->row_variant].NT;
+        const RowVariant& v = rv[is_untuned(*t) ? tv_row_default(t->W, LLONG_MAX) : t->row_variant];
+        t->rows_per_strip = v.R;
+        t->walk_depth = v.D;
+        t->row_threads = v.NT;
     } else {
         if (t->row_variant != 0) return false;
         t->rows_per_strip = haar_row_strip(t->W);
@@ -1780,6 +1786,8 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
         for (int ln : {1, kMaxLanes}) {
             if (rc != ADMM_OK || !have_win) break;
             admm_tuning_t t = win;
+            // (the untuned class with lanes set would be row configuration 0)
+            if (reg == ADMM_REG_TV && is_untuned(t)) t.row_variant = tv_row_default(W, (long long)H * W * problems);
             t.lanes = ln;
             rc = trial(t);
         }
