@@ -399,12 +399,13 @@ ADMM_API int admm_deconv_get_launch_overlap(void);
  * (device, H, W, regulariser, levels), says which configuration new plans of
  * that class use. An entry with row_variant, col_variant, slot_ctas and lanes
  * all 0 is the untuned class, as if it were not there: column index 0, 9600
- * CTAs and the row configuration that suits the width and the number of problems
- * of the call (rows_per_strip and the like describe a large batch's). Any other
- * entry fixes its row configuration, whatever the number of problems. Every
- * configuration gives the same iterates. Calls of few small TV images (sides up
- * to 256) keep each image on one team of CTAs and use the table for their layout
- * only.
+ * CTAs (3600 in a call of several classes, whose time to tolerance grows with
+ * the problems in flight) and the row configuration that suits the width and the
+ * number of problems of the call (rows_per_strip and the like describe a large
+ * batch's). Any other entry fixes its row configuration, whatever the number of
+ * problems. Every configuration gives the same iterates. Calls of few small TV
+ * images (sides up to 256) keep each image on one team of CTAs and use the table
+ * for their layout only.
  * Plans keep the configuration they were created with, and a batch groups
  * plans by shape AND configuration. The table is library-global. Entries are
  * per kernel family: plans of ADMM_REG_TV_ANISO use the ADMM_REG_TV entry,
@@ -417,7 +418,8 @@ typedef struct {
     int    row_variant;     /* index of the TV row-phase configuration of W (0 for Haar; 0 with
                                the three fields below 0: chosen by each call)                 */
     int    col_variant;     /* index of the column-phase configuration of H                  */
-    int    slot_ctas;       /* row-side CTAs per launch aimed for (0 = default 9600)         */
+    int    slot_ctas;       /* row-side CTAs per launch aimed for (0 = default 9600, or 3600
+                               in a call of several classes)                                  */
     int    lanes;           /* independent lanes (graph branches) the class's problems and
                                slots are split into, 1..4 (0 = default: 1 up to
                                2 Mpixel in flight, 2 above)                                   */

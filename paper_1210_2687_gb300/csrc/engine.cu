@@ -335,6 +335,14 @@ int gen_twiddles(DeviceCtx* c, int N, const float2** out) {
 // 1024^2 x 16 24.6 -> 24.1; frame 512^2 x 64 15.3 -> 14.7, 1024^2 x 24 64.2 ->
 // 57.7. 19200 gives no more (4.65, 1.77, 24.2; 14.5, 57.7).
 constexpr int kDefaultSlotCtas = 9600;
+// A class of a mixed call has company: the classes fill the GPU together, and
+// more problems in flight only make each take longer from its start to its
+// tolerance. So it aims for fewer, unless the rest is less than half of that
+// (those would run in launches that are half empty). 256 problems of ten classes,
+// images/s and median / 99th percentile of the time to tolerance (s): all in
+// flight 69.5, 2.60 / 3.47; 2400 CTAs 67.3, 1.37 / 2.33; 3600 68.2, 1.85 / 2.68;
+// 4200 69.5, 2.02 / 2.84; 3600 and the rest rule 69.1, 1.91 / 2.66.
+constexpr int kMixedSlotCtas = 3600;
 
 int col_block(int H) {
     const ColVariant* v = nullptr;
@@ -346,11 +354,12 @@ int row_strip_tv(int W) {
 }
 
 // launch slots of a group: enough problems in flight that a row-side launch
-// has about `slot_ctas` CTAs
-int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count) {
+// has about `slot_ctas` CTAs (0: the default; mixed: the call has other groups)
+int choose_slots(int H, int W, bool tv, int R, int slot_ctas, int count, bool mixed) {
     const int per = tv ? H / R : haar_num_tiles(H, W);
-    const int target = slot_ctas > 0 ? slot_ctas : kDefaultSlotCtas;
+    const int target = slot_ctas > 0 ? slot_ctas : mixed ? kMixedSlotCtas : kDefaultSlotCtas;
     int want = (target + per - 1) / per;
+    if (mixed && slot_ctas <= 0 && 2 * count <= 3 * want) want = count;
     if (g_max_slots > 0) want = std::min(want, g_max_slots);
     return std::max(1, std::min(count, want));
 }
@@ -1304,7 +1313,7 @@ static int solve_all_impl(DeviceCtx* ctx, const std::vector<std::vector<int>>& c
             const int r = learned();
             if (r != ADMM_OK) return learned_failed(r);
         }
-        g.nslots = choose_slots(g.H, g.W, g.tv, g.R, g.slot_ctas, g.count);
+        g.nslots = choose_slots(g.H, g.W, g.tv, g.R, g.slot_ctas, g.count, classes.size() > 1);
         // with per-phase timing on, one lane: every launch covers all slots,
         // so the timed phases are the full-size kernels
         // (as is a class that runs in teams)
