@@ -442,17 +442,23 @@ def admm_deconv_autotune(H: int, W: int, reg="tv", levels: int = 4, problems: in
     return best.as_dict(), [trials[i].as_dict() for i in range(min(n.value, cap))]
 
 
+# what an entry of the tuning cache means: 2 = defaults of 9600 CTAs and of one or two lanes by the pixels in flight,
+# all-zero entries choosing their rows by call. A cache written under another meaning is measured again.
+_TUNING_GENERATION = 2
+
+
 def tuning_cache_key(H: int, W: int, reg="tv", levels: int = 4, device_name: str = "", problems: int = 0) -> str:
     r = _REG.get(reg, reg)
     key = f"{device_name}|{int(H)}x{int(W)}|{'tv' if r == ADMM_REG_TV else 'haar'}|{0 if r == ADMM_REG_TV else int(levels) or 4}"
-    return key + (f"|p{int(problems)}" if problems > 0 else "")
+    return key + (f"|p{int(problems)}" if problems > 0 else "") + f"|g{_TUNING_GENERATION}"
 
 
 def autotune_cached(H: int, W: int, reg="tv", levels: int = 4, path: str | None = None, device_name: str = "",
                     retune: bool = False, problems: int = 0, stream=None) -> dict:
     """Install the configuration of the class from the JSON tuning cache at
-    `path` (keyed by device name, size, regulariser, levels and, when given,
-    the number of problems solved together), or autotune it (with that many
+    `path` (keyed by device name, size, regulariser, levels, when given the
+    number of problems solved together, and what the entries' defaults mean in
+    this library), or autotune it (with that many
     problems per trial; 0 = enough to fill the launches) and add it to the
     cache. Returns the installed configuration, with "source": "cache" or
     "autotune" and, after a tuning run, "trials"."""
