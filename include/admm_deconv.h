@@ -462,9 +462,11 @@ ADMM_API int admm_deconv_set_tuning(const admm_tuning_t* t);
 
 /*
  * admm_deconv_autotune -- time every combination of the class's compiled
- * configurations and slot targets {default 9600, 1200, 4800} on the current
+ * configurations and slot targets {default 9600, 2400, 4800} on the current
  * device, then 1 and 4 lanes for the fastest of those, and install the
- * fastest. Each trial creates `problems` plans of the
+ * fastest. A combination that comes to the launches of an earlier one (all of
+ * `problems` in flight under two targets) is listed with that one's figure. Each
+ * other trial creates `problems` plans of the
  * class on a synthetic observation (9 x 9 box blur, valid-region mask, rel-x
  * rule with tolerance 0 checked every 10 iterations, so no problem retires
  * early), runs `iters` iterations of all of them once to warm up and once

@@ -1664,9 +1664,11 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
     if (rc != ADMM_OK) return rc;
     int dev = 0;
     CK(cudaGetDevice(&dev));
-    const int slot_targets[3] = {0, 1200, 4800};
+    const int slot_targets[3] = {0, 2400, 4800};
     if (problems <= 0) {
-        // enough problems that the largest slot target is filled for every row configuration
+        // enough problems that the largest slot target is filled for every row
+        // configuration (as far as 96 go)
+        const int most = std::max({kDefaultSlotCtas, slot_targets[1], slot_targets[2]});
         int need = 2;
         for (int v = 0; v < nr; ++v) {
             int per = haar_num_tiles(H, W);
@@ -1675,7 +1677,7 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
                 tv_row_variants(W, &rv);
                 per = H / rv[v].R;
             }
-            need = std::max(need, (4800 + per - 1) / per);
+            need = std::max(need, (most + per - 1) / per);
         }
         problems = std::min(need, 96);
     }
@@ -1719,6 +1721,21 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
     }
     admm_tuning_t win{};
     bool have_win = false;
+    // the launches that a trial comes to: row and column configuration, slots,
+    // lanes; and the time of each that has been measured
+    std::map<std::tuple<int, int, int, int>, double> timed;
+    auto layout = [&](const admm_tuning_t& t) {
+        int row = t.row_variant, R = 0;
+        if (reg == ADMM_REG_TV) {
+            const RowVariant* rv = nullptr;
+            tv_row_variants(W, &rv);
+            if (is_untuned(t)) row = tv_row_default(W, (long long)H * W * problems);
+            R = rv[row].R;
+        }
+        const int slots = choose_slots(H, W, reg == ADMM_REG_TV, R, t.slot_ctas, problems, false);
+        const int lanes = std::min({t.lanes > 0 ? t.lanes : default_lanes(H, W, slots), problems, slots});
+        return std::make_tuple(row, t.col_variant, slots, lanes);
+    };
     int count = 0;
     rc = ADMM_OK;
     do {
@@ -1744,6 +1761,17 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
         auto trial = [&](admm_tuning_t t) -> int {
             General general;
             describe_tuning(&t);
+            // the same launches again (a slot target that the problems do not reach, the
+            // default by another name): the figure they have, so that noise does not
+            // choose between names, and the first, the default's, stays
+            const auto key = layout(t);
+            const auto known = timed.find(key);
+            if (known != timed.end()) {
+                t.us_per_iter = known->second;
+                if (count < max_trials) trials[count] = t;
+                ++count;
+                return ADMM_OK;
+            }
             {
                 std::lock_guard<std::mutex> lk(g_mutex);
                 g_tuning[TuneKey(dev, H, W, reg, levels)] = t;
@@ -1767,6 +1795,7 @@ int admm_deconv_autotune(int H, int W, int reg, int haar_levels, int problems, i
             pls.clear();
             if (r != ADMM_OK) return r;
             t.us_per_iter = (double)ms * 1e3 / ((double)problems * (double)iters);
+            timed[key] = t.us_per_iter;
             if (count < max_trials) trials[count] = t;
             ++count;
             if (!have_win || t.us_per_iter < win.us_per_iter) {
