@@ -414,7 +414,8 @@ bool describe_tuning(admm_tuning_t* t) {
     return true;
 }
 
-// default-configuration launches (the scratch-free entry point uses these)
+// launches of the lists' first entries, whatever an untuned plan would take (the
+// scratch-free entry point uses these)
 cudaError_t launch_col(int H, const ProbDesc* d, SlotTable sl, int count, int Wc, int Wp, const float2* tw,
                        cudaStream_t s) {
     const ColVariant* v = nullptr;
@@ -993,15 +994,21 @@ int admm_deconv_set_state(admm_plan_t plan, const float* state, void* stream) {
     return ADMM_OK;
 }
 
-// Whether `count` problems of a small TV class run on teams: as many as are
-// resident at once, or twice that with clusters (a second round of teams, which
-// the hardware starts as the first ones end) where the rows are no more than
-// 128. Beyond it the general kernels, whose iteration costs about the same for
-// one image as for a few dozen, are faster. Per iteration of the whole batch,
-// team / general (us): 64 x 64: 1 image 3.9 / 17, 36: 9.0 / 18.7; 128 x 128: 4:
-// 7.3 / 17.9, 9: 9.1 / 18.8, 18 (two rounds): 16.7 / 20.2; 128 x 256: 9: 16.6 /
-// 19.5, 18: 25.7 / 24.8; 256 x 128: 9: 19.2 / 19.4, 18: 30.2 / 24.5; 256 x 256:
-// 1: 9.3 / 17.1, 2: 9.8 / 17.7.
+// Whether `count` problems of a small TV class (H rows of W) run on teams: as
+// many as are resident at once, or, with clusters and H <= 128, twice that (a
+// second round of teams, which the hardware starts as the first ones end). Beyond
+// it the general kernels, whose iteration costs about the same for one image as
+// for a few dozen, are faster. Per iteration of the whole batch (us, H x W: one
+// image; the most of one round; the most of two), team / general:
+//   64 x 64     3.8 / 13.4; 36: 5.6 / 14.9;  72: 10.7 / 17.3
+//   64 x 128    4.9 / 14.9; 36: 7.7 / 17.4;  72: 18.3 / 22.3
+//   64 x 256    6.6 / 15.5; 15: 7.0 / 17.1;  30: 13.5 / 19.1
+//   128 x 64    4.4 / 13.8; 16: 7.0 / 15.1;  36: 13.2 / 17.3
+//   128 x 128   5.7 / 15.6; 14: 7.6 / 17.0;  28: 14.8 / 18.4
+//   128 x 256   7.7 / 15.4;  7: 7.8 / 17.0;  14: 15.1 / 18.6
+//   256 x 64    6.6 / 13.8;  7: 6.7 / 14.4;  (14: 12.8 / 15.6, not taken)
+//   256 x 128   9.1 / 15.4;  7: 9.2 / 16.6;  (14: 18.0 / 17.9)
+//   256 x 256   8.3 / 15.8;  2: 8.4 / 16.2
 static bool use_tv_team(int H, int W, bool aniso, int count) {
     const int cap = tv_team_capacity(H, W, aniso);
     return count <= cap * (tv_team_cluster(H, W) && H <= 128 ? 2 : 1);

@@ -111,6 +111,7 @@ struct ProbDesc {
                               // zeta2 in d2 buffer 0; null for FS-MD and the TV priors
     int test_stall;           // test hook (ADMM_OPT_TEST_STALL): the TV row phase withholds
                               // one of its bulk copies, so that its bounded wait runs out
+                              // (a 256 x 256 image's team: one CTA gives up, team.cuh)
     const void* zmap;         // frame prior: L + 1 TMA tensor maps (128 bytes each) of the d2
                               // buffers, the synthesis tile's halo boxes (null: cp.async)
 };
